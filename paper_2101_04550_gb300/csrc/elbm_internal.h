@@ -88,6 +88,9 @@ struct Solver {
     mutable const void* tmap_f[2] = {nullptr, nullptr};
     mutable int tmap_tile_y[2] = {0, 0};
     mutable int tmap_next = 0;
+    // planes per segment of the D3Q27 single-pass launches with one and with two
+    // resident blocks per SM (0: not computed yet; segment_planes())
+    mutable int seg_planes[2] = {0, 0};
 };
 
 // One member of a batch (see batch.cuh).

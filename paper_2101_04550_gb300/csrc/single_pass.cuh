@@ -11,8 +11,8 @@
 // then the arrays swap roles.
 //
 // Geometry (D3Q27): a block of kBlock = 256 threads owns a tile of 32 x 8
-// columns and marches through a segment of kSegPlanes z planes.  Per plane k
-// it (1) requests, with cp.async, the populations of plane k+2 of its tile and
+// columns and marches through a segment of `seg` z planes.  Per plane k it
+// (1) requests, with cp.async, the populations of plane k+2 of its tile and
 // of the 80-node ring around it (2 columns x 8 and 2 rows x 32) into shared
 // memory, (2) waits for the copies of plane k+1 (requested one plane earlier)
 // and computes the anomaly of those nodes -- x and y components into a 3-deep
@@ -24,6 +24,7 @@
 // edge take the periodic image of their position: they supply the anomaly of
 // the wrapped node and relax nothing.
 #pragma once
+#include <algorithm>
 #include <utility>
 #include "step_kernels.cuh"
 
@@ -31,11 +32,52 @@ namespace elbm {
 
 constexpr int kTileX = 32, kTileY = 8;   // kTileX * kTileY == kBlock
 constexpr int kHalo = 2 * kTileX + 2 * kTileY;
-constexpr int kSegPlanes = 32;
 
 #ifndef ELBM_SINGLE_MIN_BLOCKS
 #define ELBM_SINGLE_MIN_BLOCKS 2
 #endif
+
+// Planes per segment of a D3Q27 single-pass launch.  A block marches through
+// one tile column's segment of z planes and reads two planes more than it
+// relaxes, so long segments re-read little and short ones fill the GPU.  The
+// depth (up to 64) is the one whose schedule ends first when the blocks, in
+// launch order, take the next free of `slots` resident places and a segment
+// of n planes costs n + 2.5: a march is a serial chain of planes (2.0 us each
+// for a 32 x 16 TMEM tile alone on its SM, 2.9 us under full memory traffic)
+// plus the block's start-up.  Measured with that kernel, us per step against
+// the fixed 32 planes used before: 32^3 7.1 (depth 1) against 72.5, 64^3 14.8
+// (4) against 76.2; FP16 storage 96^3 31.0 (12) against 75.9, 128^3 70.6 (29)
+// against 78.4, 160^3 125.5 (54) against 149.6; 256^3 FP32 670.4 (37) against
+// 677.2, FP16 496-500 against 512.
+inline int segment_planes(long long columns, int nz, int slots)
+{
+    int best = 1;
+    long long best_end = -1;
+    for (int seg = nz < 64 ? nz : 64; seg >= 1; --seg) {  // costs in half planes
+        const long long nseg = (nz + seg - 1) / seg, len = 2 * seg + 5, last = 2 * (nz - (nseg - 1) * seg) + 5;
+        // the full segments launch first, then one last segment per column
+        const long long full = (nseg - 1) * columns, rem = full % slots, t0 = (full / slots) * len;
+        long long end = t0 + std::max(rem ? len : 0, (columns + slots - 1) / slots * last);
+        while ((slots - rem) * ((end - t0) / last) + rem * (end - t0 >= len ? (end - t0 - len) / last : 0) < columns)
+            ++end;
+        if (best_end < 0 || end < best_end) {
+            best = seg;
+            best_end = end;
+        }
+    }
+    return best;
+}
+
+// ... of a launch over solver s in tiles of 32 x tile_y columns, per_sm blocks
+// resident on an SM (kept in the solver: the grid does not change).
+inline int solver_segment_planes(const Solver& s, int tile_y, int per_sm)
+{
+    int& seg = s.seg_planes[per_sm == 1 ? 0 : 1];
+    if (seg == 0)
+        seg = segment_planes(((s.nx + kTileX - 1) / kTileX) * ((s.ny + tile_y - 1) / tile_y), s.nz,
+                             per_sm * (s.num_sms > 0 ? s.num_sms : 152));
+    return seg;
+}
 
 // Stages hold raw storage words: the tile as [i][ty][tx] elements (rows
 // copied in 16-byte pieces when rows are 16-byte aligned), the ring as one
@@ -111,15 +153,15 @@ __device__ __forceinline__ int wrapi(int v, int n) { return v < 0 ? v + n : (v >
 __device__ __forceinline__ int modi(int v, int n) { return ((v % n) + n) % n; }
 
 template <int ST>
-__global__ void __launch_bounds__(kBlock, ELBM_SINGLE_MIN_BLOCKS) k_single_pass(StepParams p, void* dst)
+__global__ void __launch_bounds__(kBlock, ELBM_SINGLE_MIN_BLOCKS) k_single_pass(StepParams p, void* dst, int seg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SingleSmem& sm = *reinterpret_cast<SingleSmem*>(smem_raw);
     using S = Storage<ST>;
     const int tx = threadIdx.x & (kTileX - 1), ty = threadIdx.x / kTileX;
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
-    const int z0 = blockIdx.z * kSegPlanes;
-    const int z1 = min(p.nz, z0 + kSegPlanes);
+    const int z0 = blockIdx.z * seg;
+    const int z1 = min(p.nz, z0 + seg);
     const bool active = (x0 + tx < p.nx) && (y0 + ty < p.ny);
     const int gx = modi(x0 + tx, p.nx), gy = modi(y0 + ty, p.ny);  // periodic image beyond a ragged edge
     const int col_off = gx + gy * p.nx;
@@ -260,7 +302,7 @@ __device__ __forceinline__ float raw_value(const StepParams& p, typename Storage
 }
 
 template <int ST>
-__global__ void __launch_bounds__(kBlock, ELBM_SINGLE_MIN_BLOCKS) k_single_pass_fast(StepParams p, void* dst)
+__global__ void __launch_bounds__(kBlock, ELBM_SINGLE_MIN_BLOCKS) k_single_pass_fast(StepParams p, void* dst, int seg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using S = Storage<ST>;
@@ -270,8 +312,8 @@ __global__ void __launch_bounds__(kBlock, ELBM_SINGLE_MIN_BLOCKS) k_single_pass_
     constexpr int PPR = kTileX / EPC;          // pieces per tile row
     const int tx = threadIdx.x & (kTileX - 1), ty = threadIdx.x / kTileX;
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
-    const int z0 = blockIdx.z * kSegPlanes;
-    const int z1 = min(p.nz, z0 + kSegPlanes);
+    const int z0 = blockIdx.z * seg;
+    const int z1 = min(p.nz, z0 + seg);
     const int gx = x0 + tx, gy = y0 + ty;
     const int row_lo = wrapi(y0 - 1, p.ny) * p.nx + x0, row_hi = wrapi(y0 + kTileY, p.ny) * p.nx + x0;
     const T* f = static_cast<const T*>(p.f);

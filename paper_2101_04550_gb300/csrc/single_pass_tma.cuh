@@ -3,7 +3,7 @@
 //
 // What it computes is the single pass of single_pass.cuh (same tile, same
 // per-node arithmetic, bit-identical results): a block owns a tile of
-// 32 x 8 columns and marches through kSegPlanes z planes; for every plane it
+// 32 x 8 columns and marches through a segment of z planes; for every plane it
 // needs the populations of the tile and of the ring of nodes around it (for
 // the anomaly Q~ of the face neighbours, Eq. Paastar1), and the anomaly of the
 // planes above and below (own column only).
@@ -380,16 +380,16 @@ __device__ __forceinline__ void tma_tile_step(const CUtensorMap* tm_tile, const 
 }
 
 // The single-pass step of one grid on 32 x 8 tiles: block (bx, by, bz) takes
-// the tile column at (32 bx, 8 by), planes kSegPlanes bz onwards.
+// the tile column at (32 bx, 8 by), planes seg bz onwards.
 template <int ST>
 __global__ void __launch_bounds__(kTmaThreads, 2)
     k_single_pass_tma(const __grid_constant__ CUtensorMap tm_tile, const __grid_constant__ CUtensorMap tm_row,
-                      const __grid_constant__ StepParams p, void* dst)
+                      const __grid_constant__ StepParams p, void* dst, int seg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int z0 = blockIdx.z * kSegPlanes;
+    const int z0 = blockIdx.z * seg;
     tma_tile_step<ST>(&tm_tile, &tm_row, p, dst, blockIdx.x * kTileX, blockIdx.y * kTileY, z0,
-                      min(p.nz, z0 + kSegPlanes), smem_raw);
+                      min(p.nz, z0 + seg), smem_raw);
 }
 
 // TMA needs 16-byte aligned rows and whole tiles: nx a multiple of 32, ny a
@@ -432,9 +432,9 @@ cudaError_t launch_single_tma(const Solver& s, const StepParams& p, void* dst, b
     const int smem = TmaLayout<ST>::bytes;
     e = set_smem_limit_once<k_single_pass_tma<ST>>(smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTileY),
-                    (unsigned)((s.nz + kSegPlanes - 1) / kSegPlanes));
-    k_single_pass_tma<ST><<<grid, kTmaThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst);
+    const int seg = solver_segment_planes(s, kTileY, 2);
+    const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTileY), (unsigned)((s.nz + seg - 1) / seg));
+    k_single_pass_tma<ST><<<grid, kTmaThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst, seg);
     *launched = true;
     return cudaGetLastError();
 }

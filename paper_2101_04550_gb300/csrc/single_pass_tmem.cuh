@@ -3,7 +3,7 @@
 //
 // The per-node arithmetic is that of single_pass.cuh (bit-identical results).
 // A block of five warpgroups owns a tile of 32 x 16 columns and marches
-// through kSegPlanes z planes:
+// through a segment of z planes (segment_planes()):
 //   * the first warp of warpgroup 4 loads plane k of the tile with one 4-D
 //     TMA box (x 32, y 16, z 1, population 27) into a ring of tile buffers in
 //     shared memory, and the ring of nodes around the tile -- two TMA row
@@ -352,17 +352,17 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
 }
 
 // The single-pass step of one grid: block (bx, by, bz) takes the tile column
-// at (32 bx, 16 by), planes kSegPlanes bz onwards.  FX (with BC): the body
+// at (32 bx, 16 by), planes seg bz onwards.  FX (with BC): the body
 // force acts along x alone.
 template <int ST, bool BC = false, bool FX = false>
 __global__ void __launch_bounds__(kTmThreads, 1)
     k_single_pass_tmem(const __grid_constant__ CUtensorMap tm_tile, const __grid_constant__ CUtensorMap tm_row,
-                       const __grid_constant__ StepParams p, void* dst)
+                       const __grid_constant__ StepParams p, void* dst, int seg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int z0 = blockIdx.z * kSegPlanes;
+    const int z0 = blockIdx.z * seg;
     tmem_tile_step<ST, BC, FX>(&tm_tile, &tm_row, p, dst, blockIdx.x * kTileX, blockIdx.y * kTmTileY, z0,
-                               min(p.nz, z0 + kSegPlanes), smem_raw);
+                               min(p.nz, z0 + seg), smem_raw);
 }
 
 template <int ST>
@@ -383,14 +383,16 @@ cudaError_t launch_single_tmem(const Solver& s, const StepParams& p, void* dst, 
     const int smem = TmemLayout<ST>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tmem<ST, BC, FX>>(smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTmTileY),
-                    (unsigned)((s.nz + kSegPlanes - 1) / kSegPlanes));
-    // programmatic dependent launch helps the 16-bit form (+0.5 %) and costs the
-    // FP32 form 0.7 % (256^3, measured), so only 16-bit storage uses it
-    if (sizeof(typename Storage<ST>::T) == 2) {
-        e = launch_pdl(k_single_pass_tmem<ST, BC, FX>, grid, dim3(kTmThreads), smem, s.stream, tm_tile, tm_row, p, dst);
+    const int seg = solver_segment_planes(s, kTmTileY, 1);
+    const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTmTileY), (unsigned)((s.nz + seg - 1) / seg));
+    // programmatic dependent launch helps the 16-bit form at every size (256^3
+    // +0.5 %) and the FP32 form on short steps (32^3 10.3 -> 7.3 us, 128^3 94.4 ->
+    // 92.9, 160^3 187.0 -> 186.4); from 192^3 on it costs that form 0.2-0.7 %
+    if (sizeof(typename Storage<ST>::T) == 2 || s.N <= 4ll << 20) {
+        e = launch_pdl(k_single_pass_tmem<ST, BC, FX>, grid, dim3(kTmThreads), smem, s.stream, tm_tile, tm_row, p, dst,
+                       seg);
     } else {
-        k_single_pass_tmem<ST, BC, FX><<<grid, kTmThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst);
+        k_single_pass_tmem<ST, BC, FX><<<grid, kTmThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst, seg);
         e = cudaGetLastError();
     }
     *launched = e == cudaSuccess;
@@ -412,8 +414,9 @@ cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
         StepParams p;
         fill_params(s, p);
         p.parity = 0;
+        const int seg = solver_segment_planes(s, kTileY, ELBM_SINGLE_MIN_BLOCKS);
         const dim3 grid((unsigned)((s.nx + kTileX - 1) / kTileX), (unsigned)((s.ny + kTileY - 1) / kTileY),
-                        (unsigned)((s.nz + kSegPlanes - 1) / kSegPlanes));
+                        (unsigned)((s.nz + seg - 1) / seg));
         const size_t smem = sizeof(SingleSmem);
         cudaError_t e = cudaSuccess;
         ELBM_DISPATCH_STORAGE(s.storage, {
@@ -437,10 +440,10 @@ cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
             if (single_fast_ok<ST>(s)) {
                 const size_t fsmem = sizeof(FastSmem<ST>);
                 e = set_smem_limit_once<k_single_pass_fast<ST>>((int)fsmem);
-                if (e == cudaSuccess) k_single_pass_fast<ST><<<grid, kBlock, fsmem, s.stream>>>(p, dst);
+                if (e == cudaSuccess) k_single_pass_fast<ST><<<grid, kBlock, fsmem, s.stream>>>(p, dst, seg);
             } else {
                 e = set_smem_limit_once<k_single_pass<ST>>((int)smem);
-                if (e == cudaSuccess) k_single_pass<ST><<<grid, kBlock, smem, s.stream>>>(p, dst);
+                if (e == cudaSuccess) k_single_pass<ST><<<grid, kBlock, smem, s.stream>>>(p, dst, seg);
             }
         });
         if (e != cudaSuccess) return e;
