@@ -311,8 +311,8 @@ void elbm_destroy(elbm_solver* s)
     if (!s) return;
     drop_graphs(s);
     // stream-ordered frees: they wait for the solver's queued work, not the device
-    for (void* ptr : {s->f, s->f2, (void*)s->q, (void*)s->status, (void*)s->mom, (void*)s->partials,
-                      (void*)s->red_out, (void*)s->progress})
+    for (void* ptr : {s->f, s->f2, (void*)s->q, (void*)s->status, (void*)s->vel, (void*)s->partials,
+                      (void*)s->red_out, (void*)s->factors, (void*)s->progress})
         if (ptr) cudaFreeAsync(ptr, s->stream);
     delete s;
 }
@@ -607,20 +607,17 @@ int elbm_set_populations(elbm_solver* s, const void* f, int dtype, int on_device
 static cudaError_t ensure_reduce_scratch(elbm_solver* s)
 {
     cudaError_t e = cudaSuccess;
-    if (!s->mom) {
+    if (!s->partials) {
         s->red_blocks = std::max(1, std::min(8 * s->num_sms, (int)((s->N + 255) / 256)));
-        e = cudaMallocAsync((void**)&s->mom, 5 * sizeof(float) * (size_t)s->N, s->stream);
-        if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->partials, sizeof(double) * ELBM_NRED * s->red_blocks, s->stream);
+        const size_t rows = 2 * (size_t)s->red_blocks;
+        e = cudaMallocAsync((void**)&s->partials, sizeof(double) * ELBM_NRED * rows, s->stream);
         if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->red_out, sizeof(double) * ELBM_NRED, s->stream);
         if (e != cudaSuccess) {
-            if (s->mom) cudaFreeAsync(s->mom, s->stream);
             if (s->partials) cudaFreeAsync(s->partials, s->stream);
-            if (s->red_out) cudaFreeAsync(s->red_out, s->stream);
-            s->mom = nullptr;
             s->partials = s->red_out = nullptr;
             return e;
         }
-        s->bytes += 5 * sizeof(float) * (size_t)s->N + sizeof(double) * ELBM_NRED * (s->red_blocks + 1);
+        s->bytes += sizeof(double) * ELBM_NRED * (rows + 1);
     }
     return e;
 }
@@ -631,6 +628,12 @@ int elbm_reduce(elbm_solver* s, double* out)
     if (!s || !out) return fail(ELBM_ERR_ARG, "NULL argument");
     if (!s->initialised) return fail(ELBM_ERR_STATE, "elbm_reduce before init");
     cudaError_t e = ensure_reduce_scratch(s);
+    if (e == cudaSuccess && !s->vel) {
+        const size_t bytes = sizeof(float) * s->D * (size_t)s->N;
+        e = cudaMallocAsync((void**)&s->vel, bytes, s->stream);
+        if (e != cudaSuccess) s->vel = nullptr;
+        else s->bytes += bytes;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "elbm_reduce scratch");
     e = (s->D == 2) ? elbm::reduce_impl<2>(*s, &s->launches) : elbm::reduce_impl<3>(*s, &s->launches);
     if (e == cudaSuccess)
@@ -652,6 +655,12 @@ int elbm_mode_sums(elbm_solver* s, const double* k, const double* dir, double* o
     for (int a = 0; a < 3; ++a)
         if (!std::isfinite(k[a]) || !std::isfinite(dir[a])) return fail(ELBM_ERR_ARG, "k and dir must be finite");
     cudaError_t e = ensure_reduce_scratch(s);
+    if (e == cudaSuccess && !s->factors) {
+        const size_t bytes = 2 * sizeof(double) * ((size_t)s->nx + s->ny + s->nz);
+        e = cudaMallocAsync((void**)&s->factors, bytes, s->stream);
+        if (e != cudaSuccess) s->factors = nullptr;
+        else s->bytes += bytes;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "elbm_mode_sums scratch");
     e = (s->D == 2) ? elbm::mode_sums_impl<2>(*s, k, dir, &s->launches)
                     : elbm::mode_sums_impl<3>(*s, k, dir, &s->launches);

@@ -72,9 +72,10 @@ struct Solver {
     cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};  // graph-pipelined step per parity
     int graph_nodes = 0;
     int* status = nullptr;            // device status word
-    float* mom = nullptr;             // reduction scratch: rho, u[3], fmin per node
-    double* partials = nullptr;       // reduction scratch: per-block FP64 partial sums
+    float* vel = nullptr;             // reduction scratch: the velocity field
+    double* partials = nullptr;       // reduction scratch: per-block FP64 partial sums (2 red_blocks rows)
     double* red_out = nullptr;        // device copy of the ELBM_NRED results
+    double* factors = nullptr;        // mode projection scratch: a complex factor per node of each axis
     double host_red[ELBM_NRED] = {};  // host copy of the results
     int red_blocks = 0;
     long long steps_done = 0;

@@ -3,6 +3,7 @@
 #include "single_pass_d2q9.cuh"
 #include "graph_step.cuh"
 #include "batch.cuh"
+#include "diagnostics.cuh"
 
 namespace elbm {
 template cudaError_t step_two_pass_impl<2>(const Solver&, int, long long*);

@@ -3,6 +3,7 @@
 #include "single_pass_tmem.cuh"
 #include "graph_step.cuh"
 #include "batch.cuh"
+#include "diagnostics.cuh"
 #include "batch_single.cuh"
 #include "fused_aa.cuh"
 

@@ -82,14 +82,10 @@ __device__ __forceinline__ int fast_div(int n, unsigned m, int s)
 }
 
 template <int D>
-__device__ __forceinline__ Node make_node(const StepParams& p, int cell)
+__device__ __forceinline__ Node make_node_at(const StepParams& p, int x, int y, int z)
 {
     Node n;
-    n.cell = cell;
-    const int z = (D == 3) ? fast_div(cell, p.div_plane_m, p.div_plane_s) : 0;
-    const int r = cell - z * p.plane;
-    const int y = fast_div(r, p.div_nx_m, p.div_nx_s);
-    const int x = r - y * p.nx;
+    n.cell = x + y * p.nx + z * p.plane;
     n.ox[1] = x;
     n.ox[0] = (x == 0) ? p.nx - 1 : x - 1;
     n.ox[2] = (x == p.nx - 1) ? 0 : x + 1;
@@ -106,6 +102,15 @@ __device__ __forceinline__ Node make_node(const StepParams& p, int cell)
         n.oz[0] = n.oz[1] = n.oz[2] = 0;
     }
     return n;
+}
+
+template <int D>
+__device__ __forceinline__ Node make_node(const StepParams& p, int cell)
+{
+    const int z = (D == 3) ? fast_div(cell, p.div_plane_m, p.div_plane_s) : 0;
+    const int r = cell - z * p.plane;
+    const int y = fast_div(r, p.div_nx_m, p.div_nx_s);
+    return make_node_at<D>(p, r - y * p.nx, y, z);
 }
 
 // ------------------------------------------------------- AA-pattern streaming

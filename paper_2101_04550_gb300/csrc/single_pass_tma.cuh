@@ -27,8 +27,6 @@
 #pragma once
 #include <cuda.h>
 
-#include <atomic>
-
 #include "single_pass.cuh"
 
 namespace elbm {
@@ -404,22 +402,6 @@ bool single_tma_ok(const Solver& s, const void* src, const void* dst)
 // the tile (32 x tile_y x 1 x 27) and of one ring row (32 x 1 x 1 x 27);
 // cached in the solver per array and tile height.
 cudaError_t encode_population_maps(const Solver& s, const void* f, int tile_y, CUtensorMap* tile, CUtensorMap* row);
-
-// Raise kernel K's dynamic shared-memory limit to `bytes`, once per device
-// and process.
-template <auto K>
-cudaError_t set_smem_limit_once(int bytes)
-{
-    static std::atomic<unsigned long long> done{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const unsigned long long bit = 1ull << (dev & 63);
-    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
-    return e;
-}
 
 template <int ST>
 cudaError_t launch_single_tma(const Solver& s, const StepParams& p, void* dst, bool* launched)

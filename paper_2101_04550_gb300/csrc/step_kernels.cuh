@@ -3,7 +3,6 @@
 // streaming parity PAR.  Included by one translation unit per lattice.
 #pragma once
 #include <type_traits>
-#include <cfloat>
 
 #include "lbm_device.cuh"
 
@@ -320,9 +319,9 @@ cudaError_t moments_impl(const Solver& s, void* rho, void* u, int dtype, long lo
     return cudaGetLastError();
 }
 
-// Post-streaming population i of a node, unshifted, in FP64.
-template <int D, int ST>
-__device__ __forceinline__ double load_f64(const StepParams& p, const Node& n, int i)
+// Post-streaming population i of a node, unshifted, in FP32 or FP64.
+template <int D, int ST, typename TOut>
+__device__ __forceinline__ TOut load_unshifted(const StepParams& p, const Node& n, int i)
 {
     using S = Storage<ST>;
     const typename S::T* f = static_cast<const typename S::T*>(p.f);
@@ -330,19 +329,28 @@ __device__ __forceinline__ double load_f64(const StepParams& p, const Node& n, i
     const float v = S::load(f + read_slot<D>(n, p.N, i, p.parity, walls));
     // a bounced slot holds population opp(i), stored against its own baseline
     const int b = (p.parity == 1 && walls && read_bounced(n, i)) ? Lat<D>::Q - 1 - i : i;
-    return S::shifted ? (double)v + (double)p.bw[b] * (double)p.rho_ref : (double)v;
+    if (!S::shifted) return (TOut)v;
+    if (sizeof(TOut) == 4) return (TOut)fmaf(p.bw[b], p.rho_ref, v);
+    return (TOut)((double)v + (double)p.bw[b] * (double)p.rho_ref);
 }
 
 // Unshifted post-streaming populations f_i = g_i + w_i rho_ref, layout f[i][cell].
+// FP32 output of the read-out (and FP32 input of k_set_f below) takes one fused
+// multiply-add instead of an FP64 sum rounded to FP32.  Bound by HBM: 27 loads
+// and 27 stores a node, all loads in flight before the first store (FP32 storage
+// and fields, 135 x 121 x 150: 77 us, floor 78; load and store by turns, as
+// the compiler must order them when the arrays may alias, took 128).
 template <int D, int ST, typename TOut>
 __global__ void __launch_bounds__(kBlock) k_get_f(StepParams p, TOut* out)
 {
     const int cell = blockIdx.x * kBlock + threadIdx.x;
     if (cell >= p.N) return;
     const Node n = make_node<D>(p, cell);
+    TOut v[Lat<D>::Q];  // every load before the first store, which might alias
 #pragma unroll
-    for (int i = 0; i < Lat<D>::Q; ++i)
-        out[(size_t)i * p.N + cell] = (TOut)load_f64<D, ST>(p, n, i);
+    for (int i = 0; i < Lat<D>::Q; ++i) v[i] = load_unshifted<D, ST, TOut>(p, n, i);
+#pragma unroll
+    for (int i = 0; i < Lat<D>::Q; ++i) out[(size_t)i * p.N + cell] = v[i];
 }
 
 // Store caller populations at the even-parity slots.
@@ -353,11 +361,16 @@ __global__ void __launch_bounds__(kBlock) k_set_f(StepParams p, const TIn* in)
     const int cell = blockIdx.x * kBlock + threadIdx.x;
     if (cell >= p.N) return;
     typename S::T* f = static_cast<typename S::T*>(p.f);
+    TIn v[Lat<D>::Q];
+#pragma unroll
+    for (int i = 0; i < Lat<D>::Q; ++i) v[i] = in[(size_t)i * p.N + cell];
 #pragma unroll
     for (int i = 0; i < Lat<D>::Q; ++i) {
-        const double v = (double)in[(size_t)i * p.N + cell];
-        const double stored = S::shifted ? v - (double)p.bw[i] * (double)p.rho_ref : v;
-        S::store(f + i * p.N + cell, (float)stored);
+        float stored = (float)v[i];
+        if (S::shifted)
+            stored = sizeof(TIn) == 4 ? fmaf(-p.bw[i], p.rho_ref, (float)v[i])
+                                      : (float)((double)v[i] - (double)p.bw[i] * (double)p.rho_ref);
+        S::store(f + i * p.N + cell, stored);
     }
 }
 
@@ -386,277 +399,6 @@ cudaError_t set_populations_impl(const Solver& s, const void* f, int dtype, long
         else k_set_f<D, ST, float><<<grid, kBlock, 0, s.stream>>>(p, (const float*)f);
         ++*launches;
     });
-    return cudaGetLastError();
-}
-
-// ------------------------------------------------------- FP64 diagnostics
-// Stage 1: per node rho, u and min_i f_i (FP32, the step kernels' sums) into
-// scratch mom[5][N].
-template <int D, int ST>
-__global__ void __launch_bounds__(kBlock) k_red_nodes(StepParams p, float* mom)
-{
-    const int cell = blockIdx.x * kBlock + threadIdx.x;
-    if (cell >= p.N) return;
-    const Node n = make_node<D>(p, cell);
-    float g[Lat<D>::Q];
-    gather_any<D, ST>(p, n, g);
-    float drho, j[3];
-    moments<D>(p, g, drho, j);
-    float fmin = FLT_MAX;
-#pragma unroll
-    for (int i = 0; i < Lat<D>::Q; ++i) fmin = fminf(fmin, fmaf(p.bw[i], p.rho_ref, g[i]));
-    const float r = p.rho_ref + drho;
-    const float inv_r = 1.0f / r;
-    mom[cell] = r;
-    mom[(size_t)p.N + cell] = j[0] * inv_r + 0.5f * p.g[0];
-    mom[(size_t)2 * p.N + cell] = j[1] * inv_r + 0.5f * p.g[1];
-    mom[(size_t)3 * p.N + cell] = (D == 3) ? j[2] * inv_r + 0.5f * p.g[2] : 0.f;
-    mom[(size_t)4 * p.N + cell] = fmin;
-}
-
-__device__ __forceinline__ double warp_sum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_min(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_down_sync(0xffffffffu, v, o));
-    return v;
-}
-__device__ __forceinline__ double warp_max(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// Reduce ELBM_NRED FP64 accumulators over a block: warp shuffles, then one
-// shared-memory stage across the block's warps.  Result valid in thread 0.
-__device__ __forceinline__ void block_reduce(double* acc, double* out)
-{
-    __shared__ double sh[kBlock / 32][ELBM_NRED];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < ELBM_NRED; ++k) {
-        const double v = (k == 9) ? warp_min(acc[k]) : (k == 11) ? warp_max(acc[k]) : warp_sum(acc[k]);
-        if (lane == 0) sh[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < ELBM_NRED) {
-        const int k = threadIdx.x;
-        double v = sh[0][k];
-        for (int w = 1; w < kBlock / 32; ++w)
-            v = (k == 9) ? fmin(v, sh[w][k]) : (k == 11) ? fmax(v, sh[w][k]) : v + sh[w][k];
-        out[k] = v;
-    }
-}
-
-// Compensated FP32 sum: hi + lo carries the running sum to about twice FP32's
-// precision -- each addition is split exactly into its rounded sum and the
-// rounding error (Knuth's TwoSum error-free transformation), and the errors
-// accumulate in lo.  For the few dozen terms a thread adds, hi + lo is within
-// about n 2^-48 of the exact sum, so per-thread partial sums keep FP64-grade
-// accuracy while the arithmetic stays on the FP32 pipes (FP64 issue is far
-// slower on this GPU); the sums across threads and blocks are FP64.
-struct Sum2f {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = hi + x;
-        const float bp = s - hi;
-        const float err = (hi - (s - bp)) + (x - bp);
-        hi = s;
-        lo += err;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
-// Stage 2: per-block FP64 partial sums (grid-stride over nodes, compensated
-// FP32 within a thread); vorticity and d_x u_x by central differences with
-// node spacing lam.  With walls the
-// velocity beyond a wall is the negated value of the wall-adjacent node
-// (no slip half-way between the nodes), and the wall-normal gradient of u_x
-// at each wall node comes from the quadratic through the wall (u = 0, a
-// distance lam_y/2 away) and the first two nodes: (9 u_x(1st) - u_x(2nd)) / (3 lam_y).
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_red_sum(StepParams p, const float* mom, double* partials)
-{
-    Sum2f sum[ELBM_NRED];  // entries 9 (min) and 11 (max) unused
-    float fmin_ = FLT_MAX, umax = 0.f;
-    int nonfinite = 0;
-    const float* ux = mom + p.N;
-    const float* uy = mom + 2 * (size_t)p.N;
-    const float* uz = mom + 3 * (size_t)p.N;
-    const float ix = 0.5f / p.lam[0], iy = 0.5f / p.lam[1], iz = 0.5f / p.lam[2];
-    for (int cell = blockIdx.x * kBlock + threadIdx.x; cell < p.N; cell += gridDim.x * kBlock) {
-        const Node n = make_node<D>(p, cell);
-        const float r = mom[cell];
-        const float u0 = ux[cell], u1 = uy[cell], u2 = uz[cell];
-        const float uu = u0 * u0 + u1 * u1 + u2 * u2;
-        const bool finite = isfinite(r) && isfinite(uu);
-        const bool walls = p.walls_y != 0;
-        auto dy = [&](const float* v) {
-            const float up = (walls && n.yhi) ? -v[cell] : v[n.at(0, 1, 0)];
-            const float dn = (walls && n.ylo) ? -v[cell] : v[n.at(0, -1, 0)];
-            return (up - dn) * iy;
-        };
-        const float dxuy = (uy[n.at(1, 0, 0)] - uy[n.at(-1, 0, 0)]) * ix;
-        const float dyux = dy(ux);
-        float w2 = (dxuy - dyux) * (dxuy - dyux);
-        if (walls && (n.ylo || n.yhi)) {
-            const float second = n.ylo ? ux[n.at(0, 1, 0)] : ux[n.at(0, -1, 0)];
-            sum[12].add((9.0f * u0 - second) * (1.0f / (3.0f * p.lam[1])));
-        }
-        if (D == 3) {
-            const float dyuz = dy(uz);
-            const float dzuy = (uy[n.at(0, 0, 1)] - uy[n.at(0, 0, -1)]) * iz;
-            const float dzux = (ux[n.at(0, 0, 1)] - ux[n.at(0, 0, -1)]) * iz;
-            const float dxuz = (uz[n.at(1, 0, 0)] - uz[n.at(-1, 0, 0)]) * ix;
-            w2 += (dyuz - dzuy) * (dyuz - dzuy) + (dzux - dxuz) * (dzux - dxuz);
-        }
-        const float dxux = (ux[n.at(1, 0, 0)] - ux[n.at(-1, 0, 0)]) * ix;
-        sum[0].add(r);
-        sum[1].add(r * u0);
-        sum[2].add(r * u1);
-        sum[3].add(r * u2);
-        sum[4].add(r * uu);
-        sum[5].add(uu);
-        sum[6].add(w2);
-        sum[7].add(dxux * dxux);
-        sum[8].add(u0 * u0);
-        fmin_ = fminf(fmin_, mom[4 * (size_t)p.N + cell]);
-        nonfinite += finite ? 0 : 1;
-        umax = fmaxf(umax, finite ? sqrtf(uu) : 0.f);
-    }
-    double acc[ELBM_NRED];
-#pragma unroll
-    for (int k = 0; k < ELBM_NRED; ++k) acc[k] = sum[k].value();
-    acc[9] = fmin_ == FLT_MAX ? DBL_MAX : (double)fmin_;
-    acc[10] = (double)nonfinite;
-    acc[11] = (double)umax;
-    block_reduce(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
-}
-
-// Stage 3: one block folds the partials in a fixed order (deterministic).
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_red_final(const double* partials, int nblocks, double* out)
-{
-    double acc[ELBM_NRED];
-#pragma unroll
-    for (int k = 0; k < ELBM_NRED; ++k) acc[k] = 0.0;
-    acc[9] = DBL_MAX;
-    for (int b = threadIdx.x; b < nblocks; b += kBlock) {
-        const double* q = partials + (size_t)b * ELBM_NRED;
-#pragma unroll
-        for (int k = 0; k < ELBM_NRED; ++k)
-            acc[k] = (k == 9) ? fmin(acc[k], q[k]) : (k == 11) ? fmax(acc[k], q[k]) : acc[k] + q[k];
-    }
-    block_reduce(acc, out);
-}
-
-// Sums of rho and rho u_a of a caller field (FP64), for the automatic storage
-// baseline velocity: out[0] = sum rho, out[1 + a] = sum rho u_a.
-template <int D, typename TIn>
-__global__ void __launch_bounds__(kBlock) k_field_sums(int N, const TIn* rho, const TIn* u, double* partials)
-{
-    double acc[ELBM_NRED];
-#pragma unroll
-    for (int k = 0; k < ELBM_NRED; ++k) acc[k] = 0.0;
-    acc[9] = DBL_MAX;
-    for (int cell = blockIdx.x * kBlock + threadIdx.x; cell < N; cell += gridDim.x * kBlock) {
-        const double r = (double)rho[cell];
-        acc[0] += r;
-#pragma unroll
-        for (int a = 0; a < D; ++a) acc[1 + a] += r * (double)u[(size_t)a * N + cell];
-    }
-    block_reduce(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
-}
-
-template <int D>
-cudaError_t field_sums_impl(const Solver& s, const void* rho, const void* u, int dtype, long long* launches)
-{
-    if (dtype == ELBM_DTYPE_F64)
-        k_field_sums<D, double><<<s.red_blocks, kBlock, 0, s.stream>>>((int)s.N, (const double*)rho,
-                                                                      (const double*)u, s.partials);
-    else
-        k_field_sums<D, float><<<s.red_blocks, kBlock, 0, s.stream>>>((int)s.N, (const float*)rho,
-                                                                     (const float*)u, s.partials);
-    k_red_final<D><<<1, kBlock, 0, s.stream>>>(s.partials, s.red_blocks, s.red_out);
-    *launches += 2;
-    return cudaGetLastError();
-}
-
-// Shear-mode projection (the amplitude of the shear wave, Sec. III.A):
-// out[0] = sum_x (u . dir) cos(k . x), out[1] = sum_x (u . dir) sin(k . x), in
-// FP64, with x = (i lam_x, j lam_y, k lam_z) the node's physical position and
-// u the reported velocity.  The phase is reduced modulo 2 pi in FP64.
-struct ModeArgs {
-    double k[3], dir[3];
-};
-
-template <int D, int ST>
-__global__ void __launch_bounds__(kBlock) k_mode_sums(StepParams p, ModeArgs m, double* partials)
-{
-    double acc[ELBM_NRED];
-#pragma unroll
-    for (int q = 0; q < ELBM_NRED; ++q) acc[q] = 0.0;
-    acc[9] = DBL_MAX;
-    for (int cell = blockIdx.x * kBlock + threadIdx.x; cell < p.N; cell += gridDim.x * kBlock) {
-        const Node n = make_node<D>(p, cell);
-        float g[Lat<D>::Q];
-        gather_any<D, ST>(p, n, g);
-        float drho, j[3];
-        moments<D>(p, g, drho, j);
-        const float inv_r = 1.0f / (p.rho_ref + drho);
-        double us = 0.0;
-#pragma unroll
-        for (int a = 0; a < D; ++a) us += (double)(j[a] * inv_r + 0.5f * p.g[a]) * m.dir[a];
-        const int z = (D == 3) ? cell / p.plane : 0;
-        const int r = cell - z * p.plane;
-        const int y = r / p.nx, x = r - y * p.nx;
-        const double phase = m.k[0] * x * (double)p.lam[0] + m.k[1] * y * (double)p.lam[1] +
-                             (D == 3 ? m.k[2] * z * (double)p.lam[2] : 0.0);
-        double sn, cs;
-        sincos(phase, &sn, &cs);
-        acc[0] += us * cs;
-        acc[1] += us * sn;
-    }
-    block_reduce(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
-}
-
-template <int D>
-cudaError_t mode_sums_impl(const Solver& s, const double* k, const double* dir, long long* launches)
-{
-    StepParams p;
-    fill_params(s, p);
-    ModeArgs m;
-    for (int a = 0; a < 3; ++a) {
-        m.k[a] = k[a];
-        m.dir[a] = dir[a];
-    }
-    ELBM_DISPATCH_STORAGE(s.storage, {
-        k_mode_sums<D, ST><<<s.red_blocks, kBlock, 0, s.stream>>>(p, m, s.partials);
-    });
-    k_red_final<D><<<1, kBlock, 0, s.stream>>>(s.partials, s.red_blocks, s.red_out);
-    *launches += 2;
-    return cudaGetLastError();
-}
-
-template <int D>
-cudaError_t reduce_impl(const Solver& s, long long* launches)
-{
-    StepParams p;
-    fill_params(s, p);
-    const dim3 grid((unsigned)((s.N + kBlock - 1) / kBlock));
-    ELBM_DISPATCH_STORAGE(s.storage, {
-        k_red_nodes<D, ST><<<grid, kBlock, 0, s.stream>>>(p, s.mom);
-    });
-    k_red_sum<D><<<s.red_blocks, kBlock, 0, s.stream>>>(p, s.mom, s.partials);
-    k_red_final<D><<<1, kBlock, 0, s.stream>>>(s.partials, s.red_blocks, s.red_out);
-    *launches += 3;
     return cudaGetLastError();
 }
 

@@ -17,12 +17,15 @@ def _gpu():
     elbm.load()
 
 
+def field(lattice, n):
+    if lattice == elbm.D3Q27:
+        return inputs.isotropic_turbulence(n, seed=5, k0=3.0, u_rms=0.05)
+    return inputs.double_shear_layer(n, U=0.08)
+
+
 def populations(lattice, n, storage, kernel, steps, **kw):
     """Populations after the given launches of steps, from a seeded field."""
-    if lattice == elbm.D3Q27:
-        rho, u = inputs.isotropic_turbulence(n, seed=5, k0=3.0, u_rms=0.05)
-    else:
-        rho, u = inputs.double_shear_layer(n, U=0.08)
+    rho, u = field(lattice, n)
     with elbm.Solver(lattice, n, storage=storage, kernel=kernel, T=0.42, nu=0.02,
                      stream=torch.cuda.current_stream(), **kw) as s:
         s.init(rho, u)
@@ -45,3 +48,66 @@ def test_segment_depths_bitwise(n, storage):
 def test_segment_depths_of_eight_row_tiles_bitwise(n):
     want = populations(elbm.D3Q27, n, elbm.F32, 1, (3,))
     assert np.array_equal(populations(elbm.D3Q27, n, elbm.F32, 3, (3,)), want)
+
+
+# tiles of the reduction are 32 x 8 nodes, the mode sums take 32 x 64: grids
+# inside one tile, one node past it, and ragged along every axis; one array at
+# both streaming parities
+@pytest.mark.parametrize("lattice,n", [(elbm.D3Q27, (5, 3, 70)), (elbm.D3Q27, (33, 9, 3)), (elbm.D3Q27, (97, 65, 4)),
+                                       (elbm.D2Q9, (33, 5)), (elbm.D2Q9, (300, 130))])
+@pytest.mark.parametrize("steps,walls", [(0, False), (1, False), (1, True), (2, True)])
+def test_diagnostics_against_the_read_out_fields(lattice, n, steps, walls):
+    """Reductions and mode amplitude against FP64 sums over the fields that
+    elbm_moments returns.  A term of a sum carries at most 8 FP32 roundings, so
+    a sum is within 8 * 2^-24 of the sum of its terms' absolute values."""
+    lam, D = (1.0, 1.5, 2.0), 3 if lattice == elbm.D3Q27 else 2
+    rho, u = field(lattice, n)
+    with elbm.Solver(lattice, n, stretch=lam, T=0.42, nu=0.02, storage=elbm.F32_SHIFT, kernel=1, walls_y=walls,
+                     force=(1e-4, 0.0, 0.0)[:D]) as s:
+        s.init(rho, u)
+        s.step(steps)
+        red = s.reduce()
+        k = [2 * np.pi / (n[a] * lam[a]) for a in range(D)]
+        amp = s.mode_amplitude(k, (0.3, -0.8, 0.5)[:D])
+        f = s.get_populations()
+        r32, u32 = s.moments(dtype=np.float32)
+    r, v = r32.astype(np.float64), u32.astype(np.float64)
+
+    def diff(w, a):
+        ax = w.ndim - 1 - a
+        up, dn = np.roll(w, -1, ax), np.roll(w, 1, ax)
+        if walls and a == 1:
+            up = np.concatenate([np.delete(w, 0, ax), -w.take([-1], ax)], ax)
+            dn = np.concatenate([-w.take([0], ax), np.delete(w, -1, ax)], ax)
+        return (up - dn) / (2 * lam[a]), (np.abs(up) + np.abs(dn)) / (2 * lam[a])
+
+    def close(got, terms, bound=None):
+        assert abs(got - terms.sum()) <= 8 * 2.0 ** -24 * (np.abs(terms) if bound is None else bound).sum()
+
+    u2 = (v ** 2).sum(0)
+    close(red["mass"], r)
+    for a, name in enumerate(("mom_x", "mom_y", "mom_z")[:D]):
+        close(red[name], r * v[a])
+    close(red["rho_u2"], r * u2)
+    close(red["u2"], u2)
+    close(red["ux2"], v[0] ** 2)
+    pairs = [(1, 0, 0, 1)] + ([(2, 1, 1, 2), (0, 2, 2, 0)] if D == 3 else [])
+    curl, size = 0.0, 0.0
+    for a, da, b, db in pairs:
+        (x, ax_), (y, ay_) = diff(v[a], da), diff(v[b], db)
+        curl, size = curl + (x - y) ** 2, size + (ax_ + ay_) ** 2
+    close(red["curl2"], curl, size)
+    dx, size = diff(v[0], 0)
+    close(red["dxux2"], dx ** 2, size ** 2)
+    assert red["umax"] == pytest.approx(np.sqrt(u2.max()), rel=1e-6)
+    assert red["fmin"] == pytest.approx(f.min(), rel=1e-5)
+    assert red["nonfinite"] == 0
+    if walls:
+        ux = np.moveaxis(v[0], v[0].ndim - 2, 0)
+        close(red["wall_dudn"], (9 * ux[[0, -1]] - ux[[1, -2]]) / (3 * lam[1]),
+              (9 * np.abs(ux[[0, -1]]) + np.abs(ux[[1, -2]])) / (3 * lam[1]))
+    phase = sum(np.arange(n[a]).reshape([-1 if d == D - 1 - a else 1 for d in range(D)]) * lam[a] * k[a]
+                for a in range(D))
+    us = sum(v[a] * w for a, w in zip(range(D), (0.3, -0.8, 0.5)))
+    want = 2 * abs((us * np.exp(-1j * phase)).sum()) / r.size
+    assert abs(amp - want) <= 8 * 2.0 ** -24 * 2 * np.abs(us).mean() + 1e-15
