@@ -40,6 +40,10 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* map)
                  : "memory");
 }
 
+// Tile buffers of the 32-wide tiles (see launch_single_tmem()).
+template <int ST>
+constexpr int kBatchBuffers = sizeof(typename Storage<ST>::T) == 4 ? 1 : 2;
+
 // Work item: x = member, y = x0, z = y0, w = z0 | (z1 << 16).
 template <int ST, bool BC, bool FX>
 __global__ void __launch_bounds__(kTmThreads, 1)
@@ -58,8 +62,8 @@ __global__ void __launch_bounds__(kTmThreads, 1)
         tensormap_acquire(&m->maps16[a][1]);
     }
     __syncthreads();
-    tmem_tile_step<ST, BC, FX>(&m->maps16[a][0], &m->maps16[a][1], sp, m->params[a ^ 1].f, w.y, w.z, w.w & 0xffff,
-                               w.w >> 16, smem_raw);
+    tmem_tile_step<ST, kTileX, kBatchBuffers<ST>, BC, FX>(&m->maps16[a][0], &m->maps16[a][1], sp, m->params[a ^ 1].f, w.y, w.z,
+                                       w.w & 0xffff, w.w >> 16, smem_raw);
 }
 
 // The same over 32 x 8 tile columns with the TMA kernel's tile body
@@ -100,7 +104,7 @@ cudaError_t sp_batch_launch_tma(const SpMember* members, const int4* work, int n
 template <int ST, bool BC, bool FX>
 cudaError_t sp_batch_launch(const SpMember* members, const int4* work, int nwork, int nsteps, cudaStream_t st)
 {
-    const int smem = TmemLayout<ST>::bytes;
+    const int smem = TmemLayout<ST, kTileX, kBatchBuffers<ST>>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tmem_batch<ST, BC, FX>>(smem);
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         k_single_pass_tmem_batch<ST, BC, FX><<<nwork, kTmThreads, smem, st>>>(members, work, k);
@@ -135,8 +139,8 @@ cudaError_t sp_member_fill(const Solver& s, void* record, bool encode_maps)
         m->params[a].parity = 0;
         if (encode_maps) {
             cudaError_t e = cudaSuccess;
-            if (tmem) e = encode_population_maps(s, arr, kTmTileY, &m->maps16[a][0], &m->maps16[a][1]);
-            if (e == cudaSuccess && tma) e = encode_population_maps(s, arr, kTileY, &m->maps8[a][0], &m->maps8[a][1]);
+            if (tmem) e = encode_population_maps(s, arr, kTileX, kTmTileY, &m->maps16[a][0], &m->maps16[a][1]);
+            if (e == cudaSuccess && tma) e = encode_population_maps(s, arr, kTileX, kTileY, &m->maps8[a][0], &m->maps8[a][1]);
             if (e != cudaSuccess) return e;
         }
     }

@@ -120,6 +120,7 @@ void fill_params(const Solver& s, StepParams& p)
         for (int cy = 0; cy < 3; ++cy)
             p.bxy_r[cx + 3 * cy] = (float)(s.rho_ref * (double)p.base[0][cx] * (double)p.base[1][cy]);
     }
+    for (int cy = 0; cy < 3; ++cy) p.bxy_pm[cy] = make_float2(p.bxy_r[3 * cy], p.bxy_r[3 * cy + 2]);
     p.T = (float)s.T;
     p.omega = (float)s.omega;
     p.coef = (float)((2.0 - s.omega) / (2.0 * s.omega));

@@ -31,6 +31,7 @@ struct StepParams {
     float base[3][3];     // storage baseline triplet per axis: Psi_c(U0_a, T + U0_a^2, lam_a)
     float base_xr[3];     // rho_ref base[0][c]
     float bxy_r[9];       // rho_ref base[0][cx] base[1][cy], index cx + 3 cy
+    float2 bxy_pm[3];     // its entries cx = -1 and +1 of each cy
     float bw[kMaxQ];      // storage baseline b_i = prod_a base[a][c_ia+1]; stored g_i = f_i - rho_ref b_i
     float u0[3];          // baseline velocity U0 (zero unless set)
     float j0[3];          // rho_ref U0: baseline momentum
@@ -83,11 +84,11 @@ struct Solver {
     size_t bytes = 0;
     long long uid = 0;                // unique per solver of the process (never reused)
     // tensor maps of the TMA-fed single-pass kernels, cached per population
-    // array and tile height (tma_maps.cu); a map depends only on the array's
+    // array and tile shape (tma_maps.cu); a map depends only on the array's
     // address and the grid, so a cached one stays valid for that address
     alignas(64) mutable unsigned char tmap[2][2][128] = {};
     mutable const void* tmap_f[2] = {nullptr, nullptr};
-    mutable int tmap_tile_y[2] = {0, 0};
+    mutable int tmap_tile[2][2] = {};
     mutable int tmap_next = 0;
     // planes per segment of the D3Q27 single-pass launches with one and with two
     // resident blocks per SM (0: not computed yet; segment_planes())

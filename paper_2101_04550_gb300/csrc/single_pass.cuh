@@ -69,13 +69,13 @@ inline int segment_planes(long long columns, int nz, int slots)
     return best;
 }
 
-// ... of a launch over solver s in tiles of 32 x tile_y columns, per_sm blocks
-// resident on an SM (kept in the solver: the grid does not change).
-inline int solver_segment_planes(const Solver& s, int tile_y, int per_sm)
+// ... of a launch over solver s in tiles of tile_x x tile_y columns, per_sm blocks
+// resident on an SM (kept in the solver: the grid and its tiles do not change).
+inline int solver_segment_planes(const Solver& s, int tile_x, int tile_y, int per_sm)
 {
     int& seg = s.seg_planes[per_sm == 1 ? 0 : 1];
     if (seg == 0)
-        seg = segment_planes(((s.nx + kTileX - 1) / kTileX) * ((s.ny + tile_y - 1) / tile_y), s.nz,
+        seg = segment_planes((long long)((s.nx + tile_x - 1) / tile_x) * ((s.ny + tile_y - 1) / tile_y), s.nz,
                              per_sm * (s.num_sms > 0 ? s.num_sms : 152));
     return seg;
 }

@@ -177,8 +177,12 @@ __device__ __forceinline__ void tmem_load27(uint32_t t, float* v)
                  : "memory");
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r[26]) : "r"(t + 26) : "memory");
     tmem_wait_ld();
+    // the registers hold the values only after the wait: pin every use behind it
 #pragma unroll
-    for (int i = 0; i < 27; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 27; ++i) {
+        asm volatile("" : "+r"(r[i])::"memory");
+        v[i] = __uint_as_float(r[i]);
+    }
 }
 
 // Shared-memory layout (byte offsets from a 128-byte aligned base).  TMA
@@ -399,9 +403,10 @@ bool single_tma_ok(const Solver& s, const void* src, const void* dst)
 }
 
 // Tensor maps of one population array: dims (x, y, z, population), boxes of
-// the tile (32 x tile_y x 1 x 27) and of one ring row (32 x 1 x 1 x 27);
-// cached in the solver per array and tile height.
-cudaError_t encode_population_maps(const Solver& s, const void* f, int tile_y, CUtensorMap* tile, CUtensorMap* row);
+// the tile (tile_x x tile_y x 1 x 27) and of one ring row (tile_x x 1 x 1 x 27);
+// cached in the solver per array and tile shape.
+cudaError_t encode_population_maps(const Solver& s, const void* f, int tile_x, int tile_y, CUtensorMap* tile,
+                                   CUtensorMap* row);
 
 template <int ST>
 cudaError_t launch_single_tma(const Solver& s, const StepParams& p, void* dst, bool* launched)
@@ -409,12 +414,12 @@ cudaError_t launch_single_tma(const Solver& s, const StepParams& p, void* dst, b
     *launched = false;
     if (!single_tma_ok<ST>(s, p.f, dst)) return cudaSuccess;
     CUtensorMap tm_tile, tm_row;
-    cudaError_t e = encode_population_maps(s, p.f, kTileY, &tm_tile, &tm_row);
+    cudaError_t e = encode_population_maps(s, p.f, kTileX, kTileY, &tm_tile, &tm_row);
     if (e != cudaSuccess) return cudaSuccess;  // no TMA: the caller takes another single-pass kernel
     const int smem = TmaLayout<ST>::bytes;
     e = set_smem_limit_once<k_single_pass_tma<ST>>(smem);
     if (e != cudaSuccess) return e;
-    const int seg = solver_segment_planes(s, kTileY, 2);
+    const int seg = solver_segment_planes(s, kTileX, kTileY, 2);
     const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTileY), (unsigned)((s.nz + seg - 1) / seg));
     k_single_pass_tma<ST><<<grid, kTmaThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst, seg);
     *launched = true;

@@ -2,63 +2,83 @@
 // the populations parked in tensor memory (TMEM) between their two uses.
 //
 // The per-node arithmetic is that of single_pass.cuh (bit-identical results).
-// A block of five warpgroups owns a tile of 32 x 16 columns and marches
+// A block of five warpgroups owns a tile of 64 x 8 or 32 x 16 columns and marches
 // through a segment of z planes (segment_planes()):
 //   * the first warp of warpgroup 4 loads plane k of the tile with one 4-D
-//     TMA box (x 32, y 16, z 1, population 27) into a ring of tile buffers in
+//     TMA box (x, y, z 1, population 27) into a ring of one or two tile buffers in
 //     shared memory, and the ring of nodes around the tile -- two TMA row
-//     boxes and two columns of 16 nodes by cp.async -- into a ring of two
+//     boxes and the two columns by cp.async -- into a ring of two
 //     buffers; one mbarrier per buffer ("full") tracks both kinds of copy.
-//     With 16-bit storage its other three warps compute the anomaly of the
-//     ring (the row below, the row above, the two columns); with FP32 storage
-//     they idle (TMEM lane quarters follow a warp's rank within its
-//     warpgroup, so the consumers must make whole warpgroups) and the
-//     consumers share the ring out;
-//   * the 16 warps of warpgroups 0..3 each own one tile row.  For plane k a
+//     Its other three warps compute the anomaly of the ring: the row below, the
+//     row above, the two columns (TMEM lane quarters follow a warp's rank within its
+//     warpgroup, so the consumers must make whole warpgroups);
+//   * the 16 warps of warpgroups 0..3 own 32 nodes of the tile each.  For plane k a
 //     thread reads its node's 27 populations from shared memory once, hands
 //     the buffer back ("empty" mbarrier), parks the values in its TMEM lane,
-//     computes the anomaly Q~ of its node (FP32 storage: and of a share of the
-//     ring, the duty rotating over the warps from plane to plane), publishes it ("qready")
+//     computes the anomaly Q~ of its node, publishes it ("qready")
 //     and relaxes plane k-1 -- with the values parked one plane earlier --
 //     once every warp has published the anomaly of plane k-1 (the central
 //     difference of Eq. Paastar1 needs the face neighbours), pushing the 27
 //     results with coalesced stores.
-// Shared memory is kept small on purpose: an SM's shared memory and its L1
-// cache are carved from one array, and the step rate grew as the footprint
-// shrank.  A tile buffer comes back as soon as it has been read, and the
-// relaxation of the previous plane covers the next load, so FP32 storage runs
-// fastest with a single buffer; 16-bit storage (half the bytes, more
-// arithmetic per byte) with two.  There is no block-wide barrier in the loop.
+// A tile buffer comes back as soon as it has been read, and the relaxation of the
+// previous plane covers the next load.  There is no block-wide barrier in the loop.
+//
+// What bounds it: FP32 storage the memory system, with pushes that straddle tile
+// edges (see launch_single_tmem()); 16-bit storage instruction issue, about 750
+// instructions a node (824 before the relaxation took the populations in pairs and
+// the pushes one pointer per c_x; FP32 685, before 763), issued on 70 % of the cycles.
 // Every wait is bounded (2 s, or as soon as another thread of the block gave
 // up); a wait that gives up sets ELBM_ERR_TIMEOUT in the status word, and the
 // block winds down: the loader waits, again bounded, for the copies in flight,
 // and the TMEM is freed by the warp that allocated it.
 #pragma once
+#include "relax_pairs.cuh"
 #include "single_pass_tma.cuh"
 
 namespace elbm {
 
-constexpr int kTmTileY = 16;                      // tile rows (one consumer warp each)
-constexpr int kTmConsumers = kTileX * kTmTileY;   // 512 threads
+constexpr int kTmTileY = 16;                      // rows of the 32-wide tile (one consumer warp each)
+constexpr int kTmConsumers = kTileX * kTmTileY;   // 512 threads, a node of the tile each
+constexpr int kTmWarps = kTmConsumers / 32;
 constexpr int kTmThreads = kTmConsumers + 128;    // + the loading warpgroup
+// Registers per thread of the walls-and-force kernel: the block is launched with
+// kTmLaunchRegs for everyone (what its size leaves of the SM's), and the loading
+// warpgroup gives up what the consumers take, never more than that (channel 512 x 128 x
+// 256 FP32: 728 us per step without, 663 with; the periodic kernel needs no more
+// than 96 and FP16 runs 1.6 % slower with the split).
+constexpr int kTmLaunchRegs = 96, kTmLoaderRegs = 64, kTmConsumerRegs = 104;
+static_assert(kTmConsumers * kTmConsumerRegs + 128 * kTmLoaderRegs <= kTmThreads * kTmLaunchRegs,
+              "the consumers must not wait for registers that the block does not own");
+template <int N>
+__device__ __forceinline__ void setmaxnreg_dec()
+{
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void setmaxnreg_inc()
+{
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
 constexpr uint32_t kTmTmemCols = 256;             // 2 plane slots x 4 warps per lane quarter x 32
 
-template <int ST>
+// TX: tile width, 32 (x 16 rows) or 64 (x 8 rows); NT: tile buffers.
+template <int ST, int TX, int NT>
 struct TmemLayout {
     using T = typename Storage<ST>::T;
     static constexpr int es = (int)sizeof(T);
-    static constexpr int ntile = es == 4 ? 1 : 2;                    // tile buffers
-    // threads that compute the ring's anomaly apart from the consumers: for
-    // 16-bit storage (issue-bound) the three spare warps of the loading
-    // warpgroup; for FP32 (latency-bound) the consumers share it out
-    static constexpr int ring_threads = es == 4 ? 0 : 96;
-    static constexpr int tile_bytes = 27 * kTmTileY * kTileX * es;   // one plane of the tile
-    static constexpr int row_box_bytes = 27 * kTileX * es;           // one ring row, all populations
+    static constexpr int TY = kTmConsumers / TX;
+    static constexpr int ntile = NT;
+    static constexpr int ring_warps = 3;  // spare warps of the loading warpgroup, for the ring's anomaly
+    static constexpr int tile_bytes = 27 * kTmConsumers * es;   // one plane of the tile
+    static constexpr int row_box_bytes = 27 * TX * es;               // one ring row, all populations
     static constexpr int row_stride = (row_box_bytes + 127) / 128 * 128;
-    static constexpr int ncol = 2 * kTmTileY;                        // ring column nodes
+    static constexpr int ncol = 2 * TY;                        // ring column nodes
     static constexpr int cols_bytes = 27 * ncol * 4;                 // as 4-byte words
-    static constexpr int qx_bytes = kTmTileY * (kTileX + 2) * 4;
-    static constexpr int qy_bytes = (kTmTileY + 2) * kTileX * 4;
+    static constexpr int qx_bytes = TY * (TX + 2) * 4;
+    static constexpr int qy_bytes = (TY + 2) * TX * 4;
+    // the ring's anomaly in units of one warp: TX / 32 for the row below, as many
+    // for the row above, one for the two columns
+    static constexpr int row_units = TX / 32, ring_units = 2 * row_units + 1;
     static constexpr int off_tile = 0;                               // [ntile] planes
     static constexpr int off_rows = off_tile + ntile * tile_bytes;   // [2 slots][2 sides]
     static constexpr int off_cols = off_rows + 4 * row_stride;       // [2 slots]
@@ -76,23 +96,24 @@ struct TmemLayout {
     static_assert(tile_bytes % 128 == 0, "tile boxes must keep 128-byte alignment");
 };
 
-// One tile column of a single-pass step: the 32 x 16 columns at (x0, y0),
+// One tile column of a single-pass step: the TX x 512/TX columns at (x0, y0),
 // planes z0 .. z1-1, from p.f into dst; every thread of the block takes part.
 // tm_tile / tm_row are the tensor maps of p.f (kernel parameters, or device
 // memory made visible to the tensor-map proxy).  smem_raw is the block's
-// dynamic shared memory (TmemLayout<ST>::bytes).
+// dynamic shared memory (TmemLayout<ST, TX, NT>::bytes).
 // BC: walls (half-way bounce-back below y = 0 and above y = ny-1, with the
 // anomaly's negated ghost value in the central difference) and the body force,
 // read from the parameter block as in the two-pass kernels; with neither set
 // in p it computes the same bits as BC = false.
-template <int ST, bool BC, bool FX = false>
+template <int ST, int TX, int NT, bool BC, bool FX = false>
 __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const CUtensorMap* tm_row,
                                                const StepParams& p, void* dst, int x0, int y0, int z0, int z1,
                                                unsigned char* smem_raw)
 {
     using S = Storage<ST>;
     using T = typename S::T;
-    using L = TmemLayout<ST>;
+    using L = TmemLayout<ST, TX, NT>;
+    constexpr int TY = L::TY;
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t sbase = (raw_addr + 127u) & ~127u;
     unsigned char* base = smem_raw + (sbase - raw_addr);
@@ -109,6 +130,8 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
     constexpr int kLoader = kTmConsumers / 32;  // first warp of the loading warpgroup
     pdl_release();
 
+    // Every thread arrives for itself (one arrival per warp behind __syncwarp() was
+    // no faster in FP32 and 2.8 % slower in FP16, 256^3)
     if (threadIdx.x == 0) {
         for (int b = 0; b < L::ntile; ++b) {
             mbar_init(full_t(b), 1);
@@ -116,9 +139,9 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
         }
         for (int r = 0; r < 2; ++r) {
             mbar_init(full_r(r), 1 + 32);  // loader lane 0 (expect_tx) + the cp.async arrivals of its 32 lanes
-            mbar_init(empty_r(r), kTmConsumers + L::ring_threads);
+            mbar_init(empty_r(r), 32 * L::ring_warps);
         }
-        for (int s = 0; s < kTmaQSlots; ++s) mbar_init(qready(s), kTmConsumers + L::ring_threads);
+        for (int s = 0; s < kTmaQSlots; ++s) mbar_init(qready(s), kTmConsumers + 32 * L::ring_warps);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -136,13 +159,42 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
     auto wait = [&](uint32_t bar, unsigned parity) { return bounded_wait(bar, parity, abort_flag, p.status, kTmaWaitNs); };
     auto drain = [&](uint32_t bar, unsigned parity) { bounded_drain(bar, parity, kTmaWaitNs); };
     auto plane_of = [&](int k) { return wrapi(z0 - 1 + k, p.nz); };
+    float* qxs = reinterpret_cast<float*>(base + L::off_qx);
+    float* qys = reinterpret_cast<float*>(base + L::off_qy);
+    auto QX = [&](int s, int y, int x) -> float& { return qxs[(s * TY + y) * (TX + 2) + x]; };
+    auto QY = [&](int s, int y, int x) -> float& { return qys[(s * (TY + 2) + y) * TX + x]; };
+    // unit u of the ring's anomaly of plane k (one warp)
+    auto ring_unit = [&](int u, int k) {
+        const int r = k & 1, s = k % kTmaQSlots;
+        auto anomaly_of = [&](auto&& gval, float* q) {
+            float drho, j[3];
+            moments_of<3>(p, gval, drho, j);
+            const float inv_rho = 1.0f / (p.rho_ref + drho);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) q[a] = anomaly(p, a, j[a], j[a] * inv_rho);
+        };
+        float qh[3];
+        if (u < 2 * L::row_units) {
+            const int side = u / L::row_units, x = (u % L::row_units) * 32 + lane;
+            const T* row = reinterpret_cast<const T*>(base + L::off_rows + (2 * r + side) * L::row_stride) + x;
+            anomaly_of([&](int i) { return raw_value<ST>(p, row[i * TX], i); }, qh);
+            QY(s, side ? TY + 1 : 0, x) = qh[1];
+        } else if (lane < L::ncol) {
+            const unsigned* cols = reinterpret_cast<const unsigned*>(base + L::off_cols + r * L::cols_bytes) + lane;
+            const int y = lane & (TY - 1), cx = lane < TY ? wrapi(x0 - 1, p.nx) : wrapi(x0 + TX, p.nx);
+            const int idx0 = plane_of(k) * p.plane + (y0 + y) * p.nx + cx;
+            anomaly_of([&](int i) { return stage_value<ST>(p, cols[i * L::ncol], (i * p.N + idx0) & 1, i); }, qh);
+            QX(s, y, lane < TY ? 0 : TX + 1) = qh[0];
+        }
+    };
 
     if (warp >= kLoader) {
+        if (BC) setmaxnreg_dec<kTmLoaderRegs>();
         if (warp == kLoader) {
             // ---------------------------------------------------- loader
-            // ring column node kk: x0-1 for kk < 16, x0+32 for kk >= 16, row y0 + (kk & 15)
-            const int ylo = wrapi(y0 - 1, p.ny), yhi = wrapi(y0 + kTmTileY, p.ny);
-            const int cxl = wrapi(x0 - 1, p.nx), cxr = wrapi(x0 + kTileX, p.nx);
+            // ring column node kk: x0-1 for kk < TY, x0+TX for kk >= TY, row y0 + kk % TY
+            const int ylo = wrapi(y0 - 1, p.ny), yhi = wrapi(y0 + TY, p.ny);
+            const int cxl = wrapi(x0 - 1, p.nx), cxr = wrapi(x0 + TX, p.nx);
             int issued = 0;
             for (int k = 0; k < K; ++k) {
                 const int b = k % L::ntile, r = k & 1;
@@ -162,8 +214,8 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                 unsigned* cols = reinterpret_cast<unsigned*>(base + L::off_cols + r * L::cols_bytes);
                 for (int c = lane; c < 27 * L::ncol; c += 32) {
                     const int i = c / L::ncol, kk = c % L::ncol;
-                    const int idx = i * p.N + zk * p.plane + (y0 + (kk & (kTmTileY - 1))) * p.nx +
-                                    (kk < kTmTileY ? cxl : cxr);
+                    const int idx = i * p.N + zk * p.plane + (y0 + (kk & (TY - 1))) * p.nx +
+                                    (kk < TY ? cxl : cxr);
                     cp_async4(cols + c, stage_src<ST>(p, idx));
                 }
                 cp_async_mbar_arrive(full_r(r));
@@ -176,39 +228,19 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                 for (int k = max(0, issued - 2); k < issued; ++k) drain(full_r(k & 1), (k / 2) & 1);
             }
             __syncwarp();
-        } else if (L::ring_threads > 0) {
+        } else {
             // ------------------------------------------------ ring anomaly
             // warp 1 of the group: the row below the tile, warp 2: the row
-            // above, warp 3: the two columns (nodes x0-1 and x0+32 of the tile's rows)
+            // above, warp 3: the two columns
             const int duty = warp - kLoader - 1;
-            auto anomaly_of = [&](auto&& gval, float* q) {
-                float drho, j[3];
-                moments_of<3>(p, gval, drho, j);
-                const float inv_rho = 1.0f / (p.rho_ref + drho);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) q[a] = anomaly(p, a, j[a], j[a] * inv_rho);
-            };
-            float* qxs = reinterpret_cast<float*>(base + L::off_qx);
-            float* qys = reinterpret_cast<float*>(base + L::off_qy);
             for (int k = 0; k < K; ++k) {
                 const int r = k & 1, s = k % kTmaQSlots;
                 if (!__all_sync(0xffffffffu, wait(full_r(r), (k / 2) & 1))) break;
                 if (k > 0 && k < K - 1) {
-                    float qh[3];
-                    if (duty < 2) {
-                        const T* row =
-                            reinterpret_cast<const T*>(base + L::off_rows + (2 * r + duty) * L::row_stride) + lane;
-                        anomaly_of([&](int i) { return raw_value<ST>(p, row[i * kTileX], i); }, qh);
-                        qys[(s * (kTmTileY + 2) + (duty ? kTmTileY + 1 : 0)) * kTileX + lane] = qh[1];
+                    if (duty == 2) {
+                        ring_unit(L::ring_units - 1, k);
                     } else {
-                        const unsigned* cols =
-                            reinterpret_cast<const unsigned*>(base + L::off_cols + r * L::cols_bytes) + lane;
-                        const int cx = lane < kTmTileY ? wrapi(x0 - 1, p.nx) : wrapi(x0 + kTileX, p.nx);
-                        const int idx0 = plane_of(k) * p.plane + (y0 + (lane & (kTmTileY - 1))) * p.nx + cx;
-                        anomaly_of([&](int i) { return stage_value<ST>(p, cols[i * L::ncol], (i * p.N + idx0) & 1, i); },
-                                   qh);
-                        qxs[(s * kTmTileY + (lane & (kTmTileY - 1))) * (kTileX + 2) + (lane < kTmTileY ? 0 : kTileX + 1)] =
-                            qh[0];
+                        for (int h = 0; h < L::row_units; ++h) ring_unit(duty * L::row_units + h, k);
                     }
                 }
                 __syncwarp();
@@ -218,71 +250,51 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
         }
     } else {
         // ------------------------------------------------------ consumers
-        const int tx = lane, ty = warp;
+        if (BC) setmaxnreg_inc<kTmConsumerRegs>();
+        const int tx = threadIdx.x & (TX - 1), ty = threadIdx.x / TX;
         const int gx = x0 + tx, gy = y0 + ty;
         const T* tile = reinterpret_cast<const T*>(base + L::off_tile);
-        float* qxs = reinterpret_cast<float*>(base + L::off_qx);
-        float* qys = reinterpret_cast<float*>(base + L::off_qy);
-        auto QX = [&](int s, int y, int x) -> float& { return qxs[(s * kTmTileY + y) * (kTileX + 2) + x]; };
-        auto QY = [&](int s, int y, int x) -> float& { return qys[(s * (kTmTileY + 2) + y) * kTileX + x]; };
         auto anomaly_m = [&](auto&& gval, float* q, float& drho, float* j, float& inv_rho) {
             moments_of<3>(p, gval, drho, j);
             inv_rho = 1.0f / (p.rho_ref + drho);
 #pragma unroll
             for (int a = 0; a < 3; ++a) q[a] = anomaly(p, a, j[a], j[a] * inv_rho);
         };
-        auto anomaly_of = [&](auto&& gval, float* q) {
-            float drho, j[3], inv_rho;
-            anomaly_m(gval, q, drho, j, inv_rho);
-        };
         // TMEM columns of this thread: its warp's lane quarter; 32 columns per
         // warp of the quarter (warps w, w+4, w+8, w+12 share a quarter); 128 per plane slot
         const uint32_t t_own = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * 32);
         T* out = static_cast<T*>(dst);
-        const int xo[3] = {gx == 0 ? p.nx - 1 : gx - 1, gx, gx == p.nx - 1 ? 0 : gx + 1};
-        const int yo[3] = {(gy == 0 ? p.ny - 1 : gy - 1) * p.nx, gy * p.nx, (gy == p.ny - 1 ? 0 : gy + 1) * p.nx};
-        constexpr int kPlaneElems = kTmTileY * kTileX;  // stride between populations in a tile buffer
+        // push target of population i = (cx, cy, cz): one pointer per cx, which stays
+        // over the march, and one 32-bit element offset per (cy, cz)
+        T* const xp[3] = {out + (gx == 0 ? p.nx - 1 : gx - 1), out + p.N + gx,
+                          out + 2 * p.N + (gx == p.nx - 1 ? 0 : gx + 1)};
+        const int yo[3] = {(gy == 0 ? p.ny - 1 : gy - 1) * p.nx, 3 * p.N + gy * p.nx,
+                           6 * p.N + (gy == p.ny - 1 ? 0 : gy + 1) * p.nx};
+        constexpr int kPlaneElems = kTmConsumers;  // stride between populations in a tile buffer
 
         float qz_prev = 0.f, qz_cur = 0.f;
         // moments of the own node of the plane relaxed next (computed with its anomaly)
         float m_drho = 0.f, m_j[3] = {0.f, 0.f, 0.f}, m_inv_rho = 1.f;
         for (int k = 0; k < K; ++k) {
-            const int b = k % L::ntile, r = k & 1, s = k % kTmaQSlots;
-            const bool got = wait(full_t(b), (k / L::ntile) & 1) && wait(full_r(r), (k / 2) & 1);
-            if (!__all_sync(0xffffffffu, got)) break;
+            const int b = k % L::ntile, s = k % kTmaQSlots;
+            if (!__all_sync(0xffffffffu, wait(full_t(b), (k / L::ntile) & 1))) break;
             float q[3], k_drho, k_j[3], k_inv_rho;
             {
-                const T* own = tile + b * 27 * kPlaneElems + ty * kTileX + tx;
-                float g[27];
+                const T* own = tile + b * 27 * kPlaneElems + threadIdx.x;
+                float g[27];  // in pair order
 #pragma unroll
-                for (int i = 0; i < 27; ++i) g[i] = raw_value<ST>(p, own[i * kPlaneElems], i);
+                for (int i = 0; i < 27; ++i) g[pair_slot(i)] = raw_value<ST>(p, own[i * kPlaneElems], i);
+                // the parking store (unused for the outer two planes) takes every value, so
+                // the reads are complete when the buffer goes back; an arrival right behind
+                // the loads can overtake them where they queue behind the loader's copies,
+                // and the refill then lands under them
+                tmem_store27(t_own + (uint32_t)((k & 1) * 128), g);
                 mbar_arrive(empty_t(b));
-                if (k >= 1 && k < K - 1) tmem_store27(t_own + (uint32_t)((k & 1) * 128), g);
-                anomaly_m([&](int i) { return g[i]; }, q, k_drho, k_j, k_inv_rho);
+                anomaly_m([&](int i) { return g[pair_slot(i)]; }, q, k_drho, k_j, k_inv_rho);
             }
             QX(s, ty, tx + 1) = q[0];
             QY(s, ty + 1, tx) = q[1];
-            // ring share of this warp for plane k (duty rotates with k): 0 the
-            // row below the tile, 1 the row above, 2 the two columns
-            const int duty = (ty + k) & (kTmTileY - 1);
-            if (L::ring_threads == 0 && k > 0 && k < K - 1) {
-                if (duty < 2) {
-                    const T* row = reinterpret_cast<const T*>(base + L::off_rows + (2 * r + duty) * L::row_stride) + tx;
-                    float qh[3];
-                    anomaly_of([&](int i) { return raw_value<ST>(p, row[i * kTileX], i); }, qh);
-                    QY(s, duty ? kTmTileY + 1 : 0, tx) = qh[1];
-                } else if (duty == 2) {
-                    const unsigned* cols = reinterpret_cast<const unsigned*>(base + L::off_cols + r * L::cols_bytes) + tx;
-                    const int cx = tx < kTmTileY ? wrapi(x0 - 1, p.nx) : wrapi(x0 + kTileX, p.nx);
-                    const int idx0 = plane_of(k) * p.plane + (y0 + (tx & (kTmTileY - 1))) * p.nx + cx;
-                    float qh[3];
-                    anomaly_of([&](int i) { return stage_value<ST>(p, cols[i * L::ncol], (i * p.N + idx0) & 1, i); },
-                               qh);
-                    QX(s, tx & (kTmTileY - 1), tx < kTmTileY ? 0 : kTileX + 1) = qh[0];
-                }
-            }
             __syncwarp();
-            mbar_arrive(empty_r(r));
             mbar_arrive(qready(s));
             if (k == 0) {
                 qz_prev = q[2];
@@ -303,7 +315,6 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
             float g[27];
             tmem_wait_st();
             tmem_load27(t_own + (uint32_t)((kc & 1) * 128), g);
-            auto gval = [&](int i) { return g[i]; };
             const float drho = m_drho, j[3] = {m_j[0], m_j[1], m_j[2]};  // moments_of of the same values
             float d[3] = {0.f, 0.f, 0.f};
             if (p.eq_mode == 0) {
@@ -315,8 +326,9 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                 d[2] = (qz_next - qz_prev) * p.inv_2lam[2];
             }
             const int z = z0 + k - 2;
-            const int zo[3] = {wrapi(z - 1, p.nz) * p.plane, z * p.plane, wrapi(z + 1, p.nz) * p.plane};
-            int yz[9];  // push target offset of the row (y + cy, z + cz)
+            const int zo[3] = {wrapi(z - 1, p.nz) * p.plane, 9 * p.N + z * p.plane,
+                               18 * p.N + wrapi(z + 1, p.nz) * p.plane};
+            int yz[9];  // push target: element offset of the row (y + cy, z + cz) of population (-1, cy, cz)
 #pragma unroll
             for (int c = 0; c < 9; ++c) yz[c] = yo[c % 3] + zo[c / 3];
             auto put = [&](int i, float gn) {
@@ -327,12 +339,11 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                     const float vb = S::shifted ? v + bounce_rebase<3>(p, 26 - i) : v;
                     S::store(out + opaque((26 - i) * p.N) + gx + gy * p.nx + z * p.plane, vb);
                 } else {
-                    const int slot = opaque(i * p.N) + (xo[cx_of(i) + 1] + yz[(cy_of(i) + 1) + 3 * (cz_of<3>(i) + 1)]);
-                    S::store(out + slot, v);
+                    S::store(xp[cx_of(i) + 1] + yz[i / 3], v);
                 }
             };
-            // (the walls-and-force kernel recomputes it: one register fewer across the loop)
-            relax_streamed<3, false, BC, FX>(p, gval, put, drho, j, d, BC ? 0.f : m_inv_rho);
+            // (the walls-and-force kernel recomputes 1/rho: one register fewer across the loop)
+            relax_pairs<BC, FX>(p, g, put, drho, j, d, BC ? 1.0f / (p.rho_ref + drho) : m_inv_rho);
             qz_prev = qz_cur;
             qz_cur = qz_next;
             m_drho = k_drho;
@@ -352,17 +363,17 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
 }
 
 // The single-pass step of one grid: block (bx, by, bz) takes the tile column
-// at (32 bx, 16 by), planes seg bz onwards.  FX (with BC): the body
+// at (TX bx, 512/TX by), planes seg bz onwards.  FX (with BC): the body
 // force acts along x alone.
-template <int ST, bool BC = false, bool FX = false>
+template <int ST, int TX, int NT, bool BC = false, bool FX = false>
 __global__ void __launch_bounds__(kTmThreads, 1)
     k_single_pass_tmem(const __grid_constant__ CUtensorMap tm_tile, const __grid_constant__ CUtensorMap tm_row,
                        const __grid_constant__ StepParams p, void* dst, int seg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int z0 = blockIdx.z * seg;
-    tmem_tile_step<ST, BC, FX>(&tm_tile, &tm_row, p, dst, blockIdx.x * kTileX, blockIdx.y * kTmTileY, z0,
-                               min(p.nz, z0 + seg), smem_raw);
+    tmem_tile_step<ST, TX, NT, BC, FX>(&tm_tile, &tm_row, p, dst, blockIdx.x * TX, blockIdx.y * (kTmConsumers / TX), z0,
+                                   min(p.nz, z0 + seg), smem_raw);
 }
 
 template <int ST>
@@ -373,30 +384,51 @@ bool single_tmem_ok(const Solver& s, const void* src, const void* dst)
            ((uintptr_t)src % 16 == 0) && ((uintptr_t)dst % 16 == 0);
 }
 
-template <int ST, bool BC = false, bool FX = false>
-cudaError_t launch_single_tmem(const Solver& s, const StepParams& p, void* dst, bool* launched)
+template <int ST, int TX, int NT, bool BC, bool FX>
+cudaError_t launch_single_tmem_tile(const Solver& s, const StepParams& p, void* dst, bool* launched)
 {
     *launched = false;
     if (!single_tmem_ok<ST>(s, p.f, dst)) return cudaSuccess;
     CUtensorMap tm_tile, tm_row;
-    if (encode_population_maps(s, p.f, kTmTileY, &tm_tile, &tm_row) != cudaSuccess) return cudaSuccess;
-    const int smem = TmemLayout<ST>::bytes;
-    cudaError_t e = set_smem_limit_once<k_single_pass_tmem<ST, BC, FX>>(smem);
+    constexpr int TY = kTmConsumers / TX;
+    if (encode_population_maps(s, p.f, TX, TY, &tm_tile, &tm_row) != cudaSuccess) return cudaSuccess;
+    const int smem = TmemLayout<ST, TX, NT>::bytes;
+    cudaError_t e = set_smem_limit_once<k_single_pass_tmem<ST, TX, NT, BC, FX>>(smem);
     if (e != cudaSuccess) return e;
-    const int seg = solver_segment_planes(s, kTmTileY, 1);
-    const dim3 grid((unsigned)(s.nx / kTileX), (unsigned)(s.ny / kTmTileY), (unsigned)((s.nz + seg - 1) / seg));
+    const int seg = solver_segment_planes(s, TX, TY, 1);
+    const dim3 grid((unsigned)(s.nx / TX), (unsigned)(s.ny / TY), (unsigned)((s.nz + seg - 1) / seg));
     // programmatic dependent launch helps the 16-bit form at every size (256^3
     // +0.5 %) and the FP32 form on short steps (32^3 10.3 -> 7.3 us, 128^3 94.4 ->
     // 92.9, 160^3 187.0 -> 186.4); from 192^3 on it costs that form 0.2-0.7 %
     if (sizeof(typename Storage<ST>::T) == 2 || s.N <= 4ll << 20) {
-        e = launch_pdl(k_single_pass_tmem<ST, BC, FX>, grid, dim3(kTmThreads), smem, s.stream, tm_tile, tm_row, p, dst,
-                       seg);
+        e = launch_pdl(k_single_pass_tmem<ST, TX, NT, BC, FX>, grid, dim3(kTmThreads), smem, s.stream, tm_tile, tm_row, p,
+                       dst, seg);
     } else {
-        k_single_pass_tmem<ST, BC, FX><<<grid, kTmThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst, seg);
+        k_single_pass_tmem<ST, TX, NT, BC, FX><<<grid, kTmThreads, smem, s.stream>>>(tm_tile, tm_row, p, dst, seg);
         e = cudaGetLastError();
     }
     *launched = e == cudaSuccess;
     return e;
+}
+
+// Tile shape and buffers.  64-wide tiles wherever nx allows: a push along x leaves
+// 32-byte sectors at the tile's edges half written by one SM and half by another,
+// half as many of them on 64-wide tiles (a plain copy of 27 shifted populations at
+// 256^3 runs at 5.4 TB/s in 32-wide tiles, 6.1 in 64-wide ones, 6.7 unshifted).
+// A second tile buffer keeps a load in flight while the first one is read; in FP32
+// its 55 KB come out of the L1 cache, which merges the pushes of a row's two warps,
+// so only the 64-wide periodic form gains at every size, the others on grids that a
+// few planes per block cover.  us per step, one against two buffers: 256^3 FP32
+// 64-wide 643 / 617, 32-wide 679 / 734; channel 512 x 128 x 256 FP32 672 / 712;
+// 64^3 14.6 / 12.9, 32^3 7.1 / 6.5.  (Before: 32-wide tiles, one buffer, the ring's
+// anomaly on the consumers: 682; FP16 32-wide 485, now 440.)
+template <int ST, bool BC = false, bool FX = false>
+cudaError_t launch_single_tmem(const Solver& s, const StepParams& p, void* dst, bool* launched)
+{
+    constexpr bool wide_storage = sizeof(typename Storage<ST>::T) == 4;
+    if (s.nx % 64 == 0) return launch_single_tmem_tile<ST, 64, wide_storage && BC ? 1 : 2, BC, FX>(s, p, dst, launched);
+    if (wide_storage && s.N > 1 << 18) return launch_single_tmem_tile<ST, 32, 1, BC, FX>(s, p, dst, launched);
+    return launch_single_tmem_tile<ST, 32, 2, BC, FX>(s, p, dst, launched);
 }
 
 // One single-pass step from s.f into dst (D3Q27 only; the caller swaps the arrays):
@@ -414,7 +446,7 @@ cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
         StepParams p;
         fill_params(s, p);
         p.parity = 0;
-        const int seg = solver_segment_planes(s, kTileY, ELBM_SINGLE_MIN_BLOCKS);
+        const int seg = solver_segment_planes(s, kTileX, kTileY, ELBM_SINGLE_MIN_BLOCKS);
         const dim3 grid((unsigned)((s.nx + kTileX - 1) / kTileX), (unsigned)((s.ny + kTileY - 1) / kTileY),
                         (unsigned)((s.nz + seg - 1) / seg));
         const size_t smem = sizeof(SingleSmem);

@@ -111,3 +111,16 @@ def test_diagnostics_against_the_read_out_fields(lattice, n, steps, walls):
     us = sum(v[a] * w for a, w in zip(range(D), (0.3, -0.8, 0.5)))
     want = 2 * abs((us * np.exp(-1j * phase)).sum()) / r.size
     assert abs(amp - want) <= 8 * 2.0 ** -24 * 2 * np.abs(us).mean() + 1e-15
+
+
+# the 64-wide tiles (8 rows) of the TMEM single pass beside the 32-wide ones (16
+# rows), with one tile buffer and with two: one tile column that wraps onto itself,
+# a single row of tiles, sizes past 2^18 nodes; FX the force along x alone
+@pytest.mark.parametrize("n", [(64, 16, 3), (64, 48, 9), (192, 16, 5), (96, 32, 7), (160, 64, 27), (128, 128, 19)])
+@pytest.mark.parametrize("storage", [elbm.F32, elbm.F32_SHIFT, elbm.F16_SHIFT, elbm.BF16_SHIFT])
+@pytest.mark.parametrize("opts", [{}, {"walls_y": True, "force": (1e-5, 0.0, 0.0)},
+                                  {"walls_y": True, "force": (1e-5, 2e-6, -3e-6)}])
+def test_tile_shapes_bitwise(n, storage, opts):
+    kw = dict(stretch=(1.5, 1.0, 2.0), **opts)
+    want = populations(elbm.D3Q27, n, storage, 1, (1, 2), **kw)
+    assert np.array_equal(populations(elbm.D3Q27, n, storage, 3, (1, 2), **kw), want)
