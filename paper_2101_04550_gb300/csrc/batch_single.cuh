@@ -106,6 +106,7 @@ cudaError_t sp_batch_launch(const SpMember* members, const int4* work, int nwork
 {
     const int smem = TmemLayout<ST, kTileX, kBatchBuffers<ST>>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tmem_batch<ST, BC, FX>>(smem);
+    if (e == cudaSuccess && BC) e = check_launch_registers<k_single_pass_tmem_batch<ST, BC, FX>>();
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         k_single_pass_tmem_batch<ST, BC, FX><<<nwork, kTmThreads, smem, st>>>(members, work, k);
         e = cudaGetLastError();

@@ -117,6 +117,7 @@ template <int D> cudaError_t step_two_pass_impl(const Solver&, int, long long*);
 template <int D> cudaError_t step_bounded_impl(const Solver&, int, long long*);
 template <int D> cudaError_t step_single_impl(const Solver&, void*, long long*);
 template <> cudaError_t step_single_impl<2>(const Solver&, void*, long long*);  // kernels_d2q9.cu
+cudaError_t launch_single_ragged(const Solver& s, const StepParams& p, void* dst);  // single_pass_ragged.cu
 bool single_tmem_geometry(const Solver& s);
 bool fused_available(const Solver& s);
 cudaError_t step_fused_impl(const Solver& s, int parity, unsigned long long* progress, unsigned long long epoch,

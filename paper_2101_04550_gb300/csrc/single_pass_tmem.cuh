@@ -61,16 +61,21 @@ __device__ __forceinline__ void setmaxnreg_inc()
 }
 constexpr uint32_t kTmTmemCols = 256;             // 2 plane slots x 4 warps per lane quarter x 32
 
-// TX: tile width, 32 (x 16 rows) or 64 (x 8 rows); NT: tile buffers.
-template <int ST, int TX, int NT>
+// TX: tile width, 32 (x 16 rows) or 64 (x 8 rows); NT: tile buffers; PB: how a tile
+// is loaded -- 0 by TMA (whole tiles), else by cp.async in pieces of 16 or 4 bytes
+// (any grid).
+template <int ST, int TX, int NT, int PB = 0>
 struct TmemLayout {
     using T = typename Storage<ST>::T;
     static constexpr int es = (int)sizeof(T);
     static constexpr int TY = kTmConsumers / TX;
     static constexpr int ntile = NT;
     static constexpr int ring_warps = 3;  // spare warps of the loading warpgroup, for the ring's anomaly
-    static constexpr int tile_bytes = 27 * kTmConsumers * es;   // one plane of the tile
-    static constexpr int row_box_bytes = 27 * TX * es;               // one ring row, all populations
+    // elements a row takes; 16-bit rows in 4-byte words start in either half of one
+    static constexpr bool words = PB == 4 && es == 2;
+    static constexpr int RS = words ? TX + 2 : TX;
+    static constexpr int tile_bytes = (27 * TY * RS * es + 127) / 128 * 128;  // one plane of the tile
+    static constexpr int row_box_bytes = 27 * RS * es;               // one ring row, all populations
     static constexpr int row_stride = (row_box_bytes + 127) / 128 * 128;
     static constexpr int ncol = 2 * TY;                        // ring column nodes
     static constexpr int cols_bytes = 27 * ncol * 4;                 // as 4-byte words
@@ -93,7 +98,7 @@ struct TmemLayout {
     static constexpr int off_abort = off_bar + 8 * nbar;
     static constexpr int off_tmem = off_abort + 4;
     static constexpr int bytes = off_abort + 16 + 128;               // + slack for aligning the base
-    static_assert(tile_bytes % 128 == 0, "tile boxes must keep 128-byte alignment");
+    static_assert(PB != 0 || tile_bytes == 27 * kTmConsumers * es, "tile boxes must keep 128-byte alignment");
 };
 
 // One tile column of a single-pass step: the TX x 512/TX columns at (x0, y0),
@@ -105,15 +110,21 @@ struct TmemLayout {
 // anomaly's negated ghost value in the central difference) and the body force,
 // read from the parameter block as in the two-pass kernels; with neither set
 // in p it computes the same bits as BC = false.
-template <int ST, int TX, int NT, bool BC, bool FX = false>
+// PB != 0: the grid may be any; the tile's last columns and rows beyond it are
+// idle, the ring closes around the ones it has, and the four warps of the loading
+// warpgroup copy the tile with cp.async, a quarter of the populations each (no
+// tensor maps: rows need not start on 16 bytes).
+template <int ST, int TX, int NT, bool BC, bool FX = false, int PB = 0>
 __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const CUtensorMap* tm_row,
                                                const StepParams& p, void* dst, int x0, int y0, int z0, int z1,
                                                unsigned char* smem_raw)
 {
     using S = Storage<ST>;
     using T = typename S::T;
-    using L = TmemLayout<ST, TX, NT>;
-    constexpr int TY = L::TY;
+    using L = TmemLayout<ST, TX, NT, PB>;
+    constexpr int TY = L::TY, RS = L::RS;
+    // columns and rows of the tile that the grid has
+    const int w = PB == 0 ? TX : min(TX, p.nx - x0), h = PB == 0 ? TY : min(TY, p.ny - y0);
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t sbase = (raw_addr + 127u) & ~127u;
     unsigned char* base = smem_raw + (sbase - raw_addr);
@@ -134,11 +145,11 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
     // no faster in FP32 and 2.8 % slower in FP16, 256^3)
     if (threadIdx.x == 0) {
         for (int b = 0; b < L::ntile; ++b) {
-            mbar_init(full_t(b), 1);
+            mbar_init(full_t(b), PB == 0 ? 1 : 128);  // expect_tx, or the loaders' cp.async arrivals
             mbar_init(empty_t(b), kTmConsumers);
         }
         for (int r = 0; r < 2; ++r) {
-            mbar_init(full_r(r), 1 + 32);  // loader lane 0 (expect_tx) + the cp.async arrivals of its 32 lanes
+            mbar_init(full_r(r), (PB == 0 ? 1 : 0) + 32);  // loader lane 0 (expect_tx) + the cp.async arrivals of its 32 lanes
             mbar_init(empty_r(r), 32 * L::ring_warps);
         }
         for (int s = 0; s < kTmaQSlots; ++s) mbar_init(qready(s), kTmConsumers + 32 * L::ring_warps);
@@ -163,6 +174,10 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
     float* qys = reinterpret_cast<float*>(base + L::off_qy);
     auto QX = [&](int s, int y, int x) -> float& { return qxs[(s * TY + y) * (TX + 2) + x]; };
     auto QY = [&](int s, int y, int x) -> float& { return qys[(s * (TY + 2) + y) * TX + x]; };
+    // 16-bit rows copied as 4-byte words: element index of the row's first node (all
+    // populations alike up to i N), and the half word population i starts in
+    auto row_start = [&](int k, int y) { return plane_of(k) * p.plane + y * p.nx + x0; };
+    auto half_of = [&](int i, int start) { return L::words ? (start + (i & 1) * p.N) & 1 : 0; };
     // unit u of the ring's anomaly of plane k (one warp)
     auto ring_unit = [&](int u, int k) {
         const int r = k & 1, s = k % kTmaQSlots;
@@ -177,25 +192,100 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
         if (u < 2 * L::row_units) {
             const int side = u / L::row_units, x = (u % L::row_units) * 32 + lane;
             const T* row = reinterpret_cast<const T*>(base + L::off_rows + (2 * r + side) * L::row_stride) + x;
-            anomaly_of([&](int i) { return raw_value<ST>(p, row[i * TX], i); }, qh);
-            QY(s, side ? TY + 1 : 0, x) = qh[1];
-        } else if (lane < L::ncol) {
+            const int start = L::words ? row_start(k, side ? wrapi(y0 + h, p.ny) : wrapi(y0 - 1, p.ny)) : 0;
+            anomaly_of([&](int i) { return raw_value<ST>(p, row[i * RS + half_of(i, start)], i); }, qh);
+            if (PB == 0 || x < w) QY(s, side ? h + 1 : 0, x) = qh[1];
+        } else if (lane < L::ncol && (PB == 0 || (lane & (TY - 1)) < h)) {
             const unsigned* cols = reinterpret_cast<const unsigned*>(base + L::off_cols + r * L::cols_bytes) + lane;
-            const int y = lane & (TY - 1), cx = lane < TY ? wrapi(x0 - 1, p.nx) : wrapi(x0 + TX, p.nx);
+            const int y = lane & (TY - 1), cx = lane < TY ? wrapi(x0 - 1, p.nx) : wrapi(x0 + w, p.nx);
             const int idx0 = plane_of(k) * p.plane + (y0 + y) * p.nx + cx;
             anomaly_of([&](int i) { return stage_value<ST>(p, cols[i * L::ncol], (i * p.N + idx0) & 1, i); }, qh);
-            QX(s, y, lane < TY ? 0 : TX + 1) = qh[0];
+            QX(s, y, lane < TY ? 0 : w + 1) = qh[0];
         }
     };
 
     if (warp >= kLoader) {
         if (BC) setmaxnreg_dec<kTmLoaderRegs>();
-        if (warp == kLoader) {
+        const int duty = warp - kLoader - 1;  // ring anomaly: 0 the row below the tile, 1 the row above, 2 the two columns
+        auto ring_plane = [&](int k) {
+            if (k > 0 && k < K - 1) {
+                if (duty == 2) {
+                    ring_unit(L::ring_units - 1, k);
+                } else {
+                    for (int u = 0; u < L::row_units; ++u) ring_unit(duty * L::row_units + u, k);
+                }
+            }
+            __syncwarp();
+            mbar_arrive(empty_r(k & 1));
+            mbar_arrive(qready(k % kTmaQSlots));
+        };
+        // ring column node kk: x0-1 for kk < TY, x0+w for kk >= TY, row y0 + kk % TY
+        const int ylo = wrapi(y0 - 1, p.ny), yhi = wrapi(y0 + h, p.ny);
+        const int cxl = wrapi(x0 - 1, p.nx), cxr = wrapi(x0 + w, p.nx);
+        auto load_columns = [&](int zk, int r) {
+            unsigned* cols = reinterpret_cast<unsigned*>(base + L::off_cols + r * L::cols_bytes);
+            for (int c = lane; c < 27 * L::ncol; c += 32) {
+                const int i = c / L::ncol, kk = c % L::ncol, y = PB == 0 ? kk & (TY - 1) : min(kk & (TY - 1), h - 1);
+                const int idx = i * p.N + zk * p.plane + (y0 + y) * p.nx + (kk < TY ? cxl : cxr);
+                cp_async4(cols + c, stage_src<ST>(p, idx));
+            }
+            cp_async_mbar_arrive(full_r(r));
+        };
+        int issued = 0;
+        if constexpr (PB != 0) {
+            const T* f = static_cast<const T*>(p.f);
+            // rows [0, rows) of w elements, row r of population i starting at element
+            // i N + first + r nx, into dst rows of RS elements (one population)
+            auto copy_rows = [&](T* to, int i, int first, int rows) {
+                const int from = i * p.N + first;
+                if constexpr (PB == 16) {
+                    constexpr int E = 16 / L::es, PPR = TX / E;
+                    for (int c = lane; c < rows * PPR; c += 32) {
+                        const int y = c / PPR, x = c % PPR * E;
+                        if (x < w) cp_async16(to + y * RS + x, f + from + y * p.nx + x);
+                    }
+                } else if constexpr (L::es == 4) {
+                    for (int c = lane; c < rows * TX; c += 32) {
+                        const int y = c / TX, x = c % TX;
+                        if (x < w) cp_async4(reinterpret_cast<unsigned*>(to + y * RS + x), f + from + y * p.nx + x);
+                    }
+                } else {
+                    constexpr int NW = TX / 2 + 1;  // words that can hold a row
+                    for (int c = lane; c < rows * NW; c += 32) {
+                        const int y = c / NW, j = c % NW, at = from + y * p.nx;
+                        if (j < ((at & 1) + w + 1) >> 1)
+                            cp_async4(reinterpret_cast<unsigned*>(to + y * RS) + j,
+                                      static_cast<const unsigned*>(p.f) + (at >> 1) + j);
+                    }
+                }
+            };
+            for (int k = 0; k < K; ++k) {
+                const int b = k % L::ntile, r = k & 1, zk = plane_of(k);
+                bool ok = true;
+                if (k >= L::ntile) ok = wait(empty_t(b), ((k / L::ntile) - 1) & 1);
+                if (ok && warp == kLoader && k >= 2) ok = wait(empty_r(r), ((k / 2) - 1) & 1);
+                if (!__all_sync(0xffffffffu, ok)) break;
+                T* tile = reinterpret_cast<T*>(base + L::off_tile + b * L::tile_bytes);
+                for (int i = warp - kLoader; i < 27; i += 4) copy_rows(tile + i * TY * RS, i, zk * p.plane + y0 * p.nx + x0, h);
+                cp_async_mbar_arrive(full_t(b));
+                issued = k + 1;
+                if (warp == kLoader) {
+                    for (int side = 0; side < 2; ++side) {
+                        T* row = reinterpret_cast<T*>(base + L::off_rows + (2 * r + side) * L::row_stride);
+                        for (int i = 0; i < 27; ++i) copy_rows(row + i * RS, i, zk * p.plane + (side ? yhi : ylo) * p.nx + x0, 1);
+                    }
+                    load_columns(zk, r);
+                } else if (k > 0) {  // the ring of the plane before, while this one is on its way
+                    if (!__all_sync(0xffffffffu, wait(full_r(r ^ 1), ((k - 1) / 2) & 1))) break;
+                    ring_plane(k - 1);
+                }
+            }
+            if (warp != kLoader && issued == K && __all_sync(0xffffffffu, wait(full_r((K - 1) & 1), ((K - 1) / 2) & 1)))
+                ring_plane(K - 1);
+            cp_async_wait_all();
+            __syncwarp();
+        } else if (warp == kLoader) {
             // ---------------------------------------------------- loader
-            // ring column node kk: x0-1 for kk < TY, x0+TX for kk >= TY, row y0 + kk % TY
-            const int ylo = wrapi(y0 - 1, p.ny), yhi = wrapi(y0 + TY, p.ny);
-            const int cxl = wrapi(x0 - 1, p.nx), cxr = wrapi(x0 + TX, p.nx);
-            int issued = 0;
             for (int k = 0; k < K; ++k) {
                 const int b = k % L::ntile, r = k & 1;
                 bool ok = true;
@@ -211,14 +301,7 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                     tma_load_4d(sbase + L::off_rows + (2 * r + 1) * L::row_stride, tm_row, x0, yhi, zk, 0,
                                 full_r(r));
                 }
-                unsigned* cols = reinterpret_cast<unsigned*>(base + L::off_cols + r * L::cols_bytes);
-                for (int c = lane; c < 27 * L::ncol; c += 32) {
-                    const int i = c / L::ncol, kk = c % L::ncol;
-                    const int idx = i * p.N + zk * p.plane + (y0 + (kk & (TY - 1))) * p.nx +
-                                    (kk < TY ? cxl : cxr);
-                    cp_async4(cols + c, stage_src<ST>(p, idx));
-                }
-                cp_async_mbar_arrive(full_r(r));
+                load_columns(zk, r);
                 issued = k + 1;
             }
             cp_async_wait_all();
@@ -230,22 +313,9 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
             __syncwarp();
         } else {
             // ------------------------------------------------ ring anomaly
-            // warp 1 of the group: the row below the tile, warp 2: the row
-            // above, warp 3: the two columns
-            const int duty = warp - kLoader - 1;
             for (int k = 0; k < K; ++k) {
-                const int r = k & 1, s = k % kTmaQSlots;
-                if (!__all_sync(0xffffffffu, wait(full_r(r), (k / 2) & 1))) break;
-                if (k > 0 && k < K - 1) {
-                    if (duty == 2) {
-                        ring_unit(L::ring_units - 1, k);
-                    } else {
-                        for (int h = 0; h < L::row_units; ++h) ring_unit(duty * L::row_units + h, k);
-                    }
-                }
-                __syncwarp();
-                mbar_arrive(empty_r(r));
-                mbar_arrive(qready(s));
+                if (!__all_sync(0xffffffffu, wait(full_r(k & 1), (k / 2) & 1))) break;
+                ring_plane(k);
             }
         }
     } else {
@@ -270,7 +340,8 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                           out + 2 * p.N + (gx == p.nx - 1 ? 0 : gx + 1)};
         const int yo[3] = {(gy == 0 ? p.ny - 1 : gy - 1) * p.nx, 3 * p.N + gy * p.nx,
                            6 * p.N + (gy == p.ny - 1 ? 0 : gy + 1) * p.nx};
-        constexpr int kPlaneElems = kTmConsumers;  // stride between populations in a tile buffer
+        constexpr int kPlaneElems = TY * RS;  // stride between populations in a tile buffer
+        const bool active = PB == 0 || (tx < w && ty < h);
 
         float qz_prev = 0.f, qz_cur = 0.f;
         // moments of the own node of the plane relaxed next (computed with its anomaly)
@@ -280,10 +351,11 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
             if (!__all_sync(0xffffffffu, wait(full_t(b), (k / L::ntile) & 1))) break;
             float q[3], k_drho, k_j[3], k_inv_rho;
             {
-                const T* own = tile + b * 27 * kPlaneElems + threadIdx.x;
+                const T* own = tile + b * (L::tile_bytes / L::es) + ty * RS + tx;
+                const int start = L::words ? row_start(k, gy) : 0;
                 float g[27];  // in pair order
 #pragma unroll
-                for (int i = 0; i < 27; ++i) g[pair_slot(i)] = raw_value<ST>(p, own[i * kPlaneElems], i);
+                for (int i = 0; i < 27; ++i) g[pair_slot(i)] = raw_value<ST>(p, own[i * kPlaneElems + half_of(i, start)], i);
                 // the parking store (unused for the outer two planes) takes every value, so
                 // the reads are complete when the buffer goes back; an arrival right behind
                 // the loads can overtake them where they queue behind the loader's copies,
@@ -292,8 +364,10 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                 mbar_arrive(empty_t(b));
                 anomaly_m([&](int i) { return g[pair_slot(i)]; }, q, k_drho, k_j, k_inv_rho);
             }
-            QX(s, ty, tx + 1) = q[0];
-            QY(s, ty + 1, tx) = q[1];
+            if (active) {
+                QX(s, ty, tx + 1) = q[0];
+                QY(s, ty + 1, tx) = q[1];
+            }
             __syncwarp();
             mbar_arrive(qready(s));
             if (k == 0) {
@@ -343,7 +417,7 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
                 }
             };
             // (the walls-and-force kernel recomputes 1/rho: one register fewer across the loop)
-            relax_pairs<BC, FX>(p, g, put, drho, j, d, BC ? 1.0f / (p.rho_ref + drho) : m_inv_rho);
+            if (active) relax_pairs<BC, FX>(p, g, put, drho, j, d, BC ? 1.0f / (p.rho_ref + drho) : m_inv_rho);
             qz_prev = qz_cur;
             qz_cur = qz_next;
             m_drho = k_drho;
@@ -384,6 +458,25 @@ bool single_tmem_ok(const Solver& s, const void* src, const void* dst)
            ((uintptr_t)src % 16 == 0) && ((uintptr_t)dst % 16 == 0);
 }
 
+// A kernel that moves registers between its warpgroups must be launched with
+// kTmLaunchRegs a thread, or its consumers would wait for registers the block does
+// not own: checked once per kernel and device.
+template <auto K>
+cudaError_t check_launch_registers()
+{
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    cudaFuncAttributes a;
+    e = cudaFuncGetAttributes(&a, K);
+    if (e == cudaSuccess && (a.numRegs + 7) / 8 * 8 < kTmLaunchRegs) e = cudaErrorInvalidConfiguration;
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
+    return e;
+}
+
 template <int ST, int TX, int NT, bool BC, bool FX>
 cudaError_t launch_single_tmem_tile(const Solver& s, const StepParams& p, void* dst, bool* launched)
 {
@@ -394,6 +487,7 @@ cudaError_t launch_single_tmem_tile(const Solver& s, const StepParams& p, void* 
     if (encode_population_maps(s, p.f, TX, TY, &tm_tile, &tm_row) != cudaSuccess) return cudaSuccess;
     const int smem = TmemLayout<ST, TX, NT>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tmem<ST, TX, NT, BC, FX>>(smem);
+    if (e == cudaSuccess && BC) e = check_launch_registers<k_single_pass_tmem<ST, TX, NT, BC, FX>>();
     if (e != cudaSuccess) return e;
     const int seg = solver_segment_planes(s, TX, TY, 1);
     const dim3 grid((unsigned)(s.nx / TX), (unsigned)(s.ny / TY), (unsigned)((s.nz + seg - 1) / seg));
@@ -432,8 +526,8 @@ cudaError_t launch_single_tmem(const Solver& s, const StepParams& p, void* dst, 
 }
 
 // One single-pass step from s.f into dst (D3Q27 only; the caller swaps the arrays):
-// the TMA-fed kernels where the geometry allows (32 x 16 tiles with TMEM,
-// else 32 x 8 tiles), else the cp.async-staged ones.
+// the TMA-fed kernels where the geometry allows (whole tiles with TMEM, else 32 x 8
+// tiles), else the cp.async-fed TMEM one (single_pass_ragged.cu).
 template <int D>
 cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
 {
@@ -446,10 +540,6 @@ cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
         StepParams p;
         fill_params(s, p);
         p.parity = 0;
-        const int seg = solver_segment_planes(s, kTileX, kTileY, ELBM_SINGLE_MIN_BLOCKS);
-        const dim3 grid((unsigned)((s.nx + kTileX - 1) / kTileX), (unsigned)((s.ny + kTileY - 1) / kTileY),
-                        (unsigned)((s.nz + seg - 1) / seg));
-        const size_t smem = sizeof(SingleSmem);
         cudaError_t e = cudaSuccess;
         ELBM_DISPATCH_STORAGE(s.storage, {
             bool done = false;
@@ -465,22 +555,11 @@ cudaError_t step_single_impl(const Solver& s, void* dst, long long* launches)
             }
             e = launch_single_tmem<ST>(s, p, dst, &done);
             if (e == cudaSuccess && !done) e = launch_single_tma<ST>(s, p, dst, &done);
-            if (e != cudaSuccess || done) {
-                if (e == cudaSuccess) ++*launches;
-                return e;
-            }
-            if (single_fast_ok<ST>(s)) {
-                const size_t fsmem = sizeof(FastSmem<ST>);
-                e = set_smem_limit_once<k_single_pass_fast<ST>>((int)fsmem);
-                if (e == cudaSuccess) k_single_pass_fast<ST><<<grid, kBlock, fsmem, s.stream>>>(p, dst, seg);
-            } else {
-                e = set_smem_limit_once<k_single_pass<ST>>((int)smem);
-                if (e == cudaSuccess) k_single_pass<ST><<<grid, kBlock, smem, s.stream>>>(p, dst, seg);
-            }
+            if (e == cudaSuccess && !done) e = launch_single_ragged(s, p, dst);
         });
         if (e != cudaSuccess) return e;
         ++*launches;
-        return cudaGetLastError();
+        return cudaSuccess;
     }
 }
 
