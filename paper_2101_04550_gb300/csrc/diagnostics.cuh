@@ -59,34 +59,49 @@ __device__ __forceinline__ void block_reduce(const double* acc, double* out)
     }
 }
 
-// Last stage: fold the blocks' partials in a fixed order (deterministic), one
-// warp per quantity.
-constexpr int kFinalThreads = 32 * ELBM_NRED;
-template <int D>
-__global__ void __launch_bounds__(kFinalThreads) k_red_final(const double* partials, int nblocks, int nq, double* out)
+// Last stage of a reduction kernel, taken by the block that finishes last: fold the
+// partials of `rows` blocks in a fixed order (deterministic), a warp per quantity,
+// and put the solver's status word behind the ELBM_NRED results, so that one copy
+// brings both to the host.  `partials` are this kernel's own (already written by
+// every block) and, before them, those of earlier kernels on the stream; *counter is
+// zero between launches.  (A kernel of its own for this took 14 us and a launch.)
+__device__ __forceinline__ void finish_reduction(const double* partials, int rows, int nq, unsigned* counter,
+                                                 const int* status, double* out)
 {
-    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
-    if (k >= nq) return;
-    auto fold = [&](double none, auto&& op) {
-        constexpr int U = 8;  // independent chains, and loads in flight
-        double v[U];
+    __shared__ bool last;
+    __threadfence();  // this block's partials, before it counts itself done
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < nq; k += kBlock / 32) {
+        auto fold = [&](double none, auto&& op) {
+            constexpr int U = 8;  // independent chains, and loads in flight
+            double v[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) v[j] = none;
-        for (int b0 = lane; b0 < nblocks; b0 += 32 * U)
+            for (int j = 0; j < U; ++j) v[j] = none;
+            for (int b0 = lane; b0 < rows; b0 += 32 * U)
 #pragma unroll
-            for (int j = 0; j < U; ++j)
-                if (b0 + 32 * j < nblocks) v[j] = op(v[j], partials[(size_t)(b0 + 32 * j) * ELBM_NRED + k]);
+                for (int j = 0; j < U; ++j)
+                    if (b0 + 32 * j < rows) v[j] = op(v[j], __ldcg(partials + (size_t)(b0 + 32 * j) * ELBM_NRED + k));
 #pragma unroll
-        for (int w = U / 2; w > 0; w /= 2)
+            for (int w = U / 2; w > 0; w /= 2)
 #pragma unroll
-            for (int j = 0; j < w; ++j) v[j] = op(v[j], v[j + w]);
-        return v[0];
-    };
-    double v;
-    if (k == 9) v = warp_min(fold(DBL_MAX, [](double a, double b) { return fmin(a, b); }));
-    else if (k == 11) v = warp_max(fold(0.0, [](double a, double b) { return fmax(a, b); }));
-    else v = warp_sum(fold(0.0, [](double a, double b) { return a + b; }));
-    if (lane == 0) out[k] = v;
+                for (int j = 0; j < w; ++j) v[j] = op(v[j], v[j + w]);
+            return v[0];
+        };
+        double v;
+        if (k == 9) v = warp_min(fold(DBL_MAX, [](double a, double b) { return fmin(a, b); }));
+        else if (k == 11) v = warp_max(fold(0.0, [](double a, double b) { return fmax(a, b); }));
+        else v = warp_sum(fold(0.0, [](double a, double b) { return a + b; }));
+        if (lane == 0) out[k] = v;
+    }
+    if (threadIdx.x == 0) {
+        out[ELBM_NRED] = (double)*status;
+        *counter = 0;
+    }
 }
 
 // Compensated FP32 sum: hi + lo carries the running sum to about twice FP32's
@@ -172,7 +187,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_red_nodes(const __grid_constant__
 // (160 us at 256^3); four nodes share 11 16-byte loads and 6 words (90 us).
 template <int D, int V>
 __global__ void __launch_bounds__(kBlock) k_red_gradients(const __grid_constant__ StepParams p, const float* __restrict__ vel,
-                                                          double* partials)
+                                                          double* partials, int node_rows, unsigned* counter, double* out)
 {
     Sum2f curl2, dxux2, wall;
     const bool walls = p.walls_y != 0;
@@ -237,7 +252,8 @@ __global__ void __launch_bounds__(kBlock) k_red_gradients(const __grid_constant_
     acc[7] = dxux2.value();
     acc[9] = DBL_MAX;
     acc[12] = wall.value();
-    block_reduce<ELBM_NRED>(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
+    block_reduce<ELBM_NRED>(acc, partials + (size_t)(node_rows + blockIdx.x) * ELBM_NRED);
+    finish_reduction(partials, node_rows + gridDim.x, ELBM_NRED, counter, p.status, out);
 }
 
 template <int D>
@@ -251,11 +267,11 @@ cudaError_t reduce_impl(const Solver& s, long long* launches)
         k_red_nodes<D, ST><<<nodes, kBlock, 0, s.stream>>>(p, s.vel, s.partials);
     });
     const int grads = std::min(s.red_blocks, 4 * s.num_sms);
-    double* rest = s.partials + (size_t)nodes * ELBM_NRED;
-    if (s.nx % 4 == 0) k_red_gradients<D, 4><<<grads, kBlock, 0, s.stream>>>(p, s.vel, rest);
-    else k_red_gradients<D, 1><<<grads, kBlock, 0, s.stream>>>(p, s.vel, rest);
-    k_red_final<D><<<1, kFinalThreads, 0, s.stream>>>(s.partials, nodes + grads, ELBM_NRED, s.red_out);
-    *launches += 3;
+    if (s.nx % 4 == 0)
+        k_red_gradients<D, 4><<<grads, kBlock, 0, s.stream>>>(p, s.vel, s.partials, nodes, s.red_counter, s.red_out);
+    else
+        k_red_gradients<D, 1><<<grads, kBlock, 0, s.stream>>>(p, s.vel, s.partials, nodes, s.red_counter, s.red_out);
+    *launches += 2;
     return cudaGetLastError();
 }
 
@@ -263,7 +279,8 @@ cudaError_t reduce_impl(const Solver& s, long long* launches)
 // Sums of rho and rho u_a of a caller field (FP64), for the automatic storage
 // baseline velocity: out[0] = sum rho, out[1 + a] = sum rho u_a.
 template <int D, typename TIn>
-__global__ void __launch_bounds__(kBlock) k_field_sums(int N, const TIn* rho, const TIn* u, double* partials)
+__global__ void __launch_bounds__(kBlock) k_field_sums(int N, const TIn* rho, const TIn* u, double* partials,
+                                                       unsigned* counter, const int* status, double* out)
 {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int cell = blockIdx.x * kBlock + threadIdx.x; cell < N; cell += gridDim.x * kBlock) {
@@ -273,6 +290,7 @@ __global__ void __launch_bounds__(kBlock) k_field_sums(int N, const TIn* rho, co
         for (int a = 0; a < D; ++a) acc[1 + a] += r * (double)u[(size_t)a * N + cell];
     }
     block_reduce<4>(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
+    finish_reduction(partials, gridDim.x, 4, counter, status, out);
 }
 
 template <int D>
@@ -280,12 +298,13 @@ cudaError_t field_sums_impl(const Solver& s, const void* rho, const void* u, int
 {
     if (dtype == ELBM_DTYPE_F64)
         k_field_sums<D, double><<<s.red_blocks, kBlock, 0, s.stream>>>((int)s.N, (const double*)rho,
-                                                                      (const double*)u, s.partials);
+                                                                      (const double*)u, s.partials, s.red_counter,
+                                                                      s.status, s.red_out);
     else
         k_field_sums<D, float><<<s.red_blocks, kBlock, 0, s.stream>>>((int)s.N, (const float*)rho,
-                                                                     (const float*)u, s.partials);
-    k_red_final<D><<<1, kFinalThreads, 0, s.stream>>>(s.partials, s.red_blocks, 4, s.red_out);
-    *launches += 2;
+                                                                     (const float*)u, s.partials, s.red_counter,
+                                                                     s.status, s.red_out);
+    ++*launches;
     return cudaGetLastError();
 }
 
@@ -322,7 +341,7 @@ __global__ void __launch_bounds__(kBlock) k_mode_factors(StepParams p, ModeArgs 
 template <int D, int ST>
 __global__ void __launch_bounds__(kBlock, 4)
     k_mode_sums(const __grid_constant__ StepParams p, ModeArgs m, const double2* factors, int chunks, int ysegs, int items,
-                double* partials)
+                double* partials, unsigned* counter, double* out)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double acc[2] = {0.0, 0.0};
@@ -351,6 +370,7 @@ __global__ void __launch_bounds__(kBlock, 4)
         acc[1] += re * s + im * c;
     }
     block_reduce<2>(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
+    finish_reduction(partials, gridDim.x, 2, counter, p.status, out);
 }
 
 template <int D>
@@ -368,10 +388,10 @@ cudaError_t mode_sums_impl(const Solver& s, const double* k, const double* dir, 
     const int items = chunks * ysegs * s.nz, blocks = std::min(items, s.red_blocks);
     k_mode_factors<D><<<(nf + kBlock - 1) / kBlock, kBlock, 0, s.stream>>>(p, m, factors);
     ELBM_DISPATCH_STORAGE(s.storage, {
-        k_mode_sums<D, ST><<<blocks, kBlock, 0, s.stream>>>(p, m, factors, chunks, ysegs, items, s.partials);
+        k_mode_sums<D, ST><<<blocks, kBlock, 0, s.stream>>>(p, m, factors, chunks, ysegs, items, s.partials, s.red_counter,
+                                                                s.red_out);
     });
-    k_red_final<D><<<1, kFinalThreads, 0, s.stream>>>(s.partials, blocks, 2, s.red_out);
-    *launches += 3;
+    *launches += 2;
     return cudaGetLastError();
 }
 

@@ -170,18 +170,32 @@ using elbm::Solver;
 
 namespace {
 
-int check_status(elbm_solver* s)
+// Report a status word read back after the solver's work so far.
+int report_status(elbm_solver* s, int st)
 {
-    int st = 0;
-    cudaError_t e = cudaMemcpyAsync(&st, s->status, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "status read");
     if (st != 0) {
         cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
         cudaStreamSynchronize(s->stream);
         return fail(st, "a bounded device-side wait gave up (code %d); the state is undefined", st);
     }
     return ELBM_OK;
+}
+
+// Wait for the solver's stream and report its status word.
+int check_status(elbm_solver* s, const char* what)
+{
+    int st = 0;
+    cudaError_t e = cudaMemcpyAsync(&st, s->status, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_fail(e, what);
+    return report_status(s, st);
+}
+
+// Wait for a reduction's results (and the status word behind them) in s->host_red.
+cudaError_t fetch_reduction(elbm_solver* s)
+{
+    cudaError_t e = cudaMemcpyAsync(s->host_red, s->red_out, sizeof s->host_red, cudaMemcpyDeviceToHost, s->stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(s->stream) : e;
 }
 
 bool shifted_storage_mode(int storage) { return storage != ELBM_F32; }
@@ -313,7 +327,7 @@ void elbm_destroy(elbm_solver* s)
     drop_graphs(s);
     // stream-ordered frees: they wait for the solver's queued work, not the device
     for (void* ptr : {s->f, s->f2, (void*)s->q, (void*)s->status, (void*)s->vel, (void*)s->partials,
-                      (void*)s->red_out, (void*)s->factors, (void*)s->progress})
+                      (void*)s->red_out, (void*)s->red_counter, (void*)s->factors, (void*)s->progress})
         if (ptr) cudaFreeAsync(ptr, s->stream);
     delete s;
 }
@@ -433,9 +447,7 @@ int elbm_init(elbm_solver* s, const void* rho, const void* u, int dtype, int on_
         if (e == cudaSuccess)
             e = (s->D == 2) ? elbm::field_sums_impl<2>(*s, drho, du, dtype, &s->launches)
                             : elbm::field_sums_impl<3>(*s, drho, du, dtype, &s->launches);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(s->host_red, s->red_out, sizeof(double) * ELBM_NRED, cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+        if (e == cudaSuccess) e = fetch_reduction(s);
         if (e == cudaSuccess) {
             for (int a = 0; a < s->D; ++a) {
                 const double U0 = s->host_red[1 + a] / s->host_red[0];
@@ -471,7 +483,11 @@ int elbm_step(elbm_solver* s, int n)
     cudaError_t e = cudaSuccess;
     int left = n;
     while (left > 0 && e == cudaSuccess) {
-        if (kernel == 3 && s->parity == 0 && s->f2) {
+        if (kernel == 3 && s->parity == 0 && s->f2 && left > 1 && elbm::small_d2q9(*s)) {
+            // a small D2Q9 grid: every step of the call in one launch, the state stays in f
+            e = elbm::steps_small_d2q9(*s, left, &s->launches);
+            left = 0;
+        } else if (kernel == 3 && s->parity == 0 && s->f2) {
             // single pass: own-location state in f, result in f2, then swap
             e = (s->D == 2) ? elbm::step_single_impl<2>(*s, s->f2, &s->launches)
                             : elbm::step_single_impl<3>(*s, s->f2, &s->launches);
@@ -519,9 +535,7 @@ int elbm_step(elbm_solver* s, int n)
 int elbm_sync(elbm_solver* s)
 {
     if (!s) return fail(ELBM_ERR_ARG, "solver is NULL");
-    cudaError_t e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "elbm_sync");
-    return check_status(s);
+    return check_status(s, "elbm_sync");
 }
 
 int elbm_moments(elbm_solver* s, void* rho, void* u, int dtype, int on_device)
@@ -553,10 +567,11 @@ int elbm_moments(elbm_solver* s, void* rho, void* u, int dtype, int on_device)
         cudaFreeAsync(drho, s->stream);
         cudaFreeAsync(du, s->stream);
     }
-    cudaError_t e2 = cudaStreamSynchronize(s->stream);
-    if (e == cudaSuccess) e = e2;
-    if (e != cudaSuccess) return cuda_fail(e, "elbm_moments");
-    return check_status(s);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(s->stream);
+        return cuda_fail(e, "elbm_moments");
+    }
+    return check_status(s, "elbm_moments");
 }
 
 int elbm_get_populations(elbm_solver* s, void* f, int dtype, int on_device)
@@ -574,10 +589,11 @@ int elbm_get_populations(elbm_solver* s, void* f, int dtype, int on_device)
                         : elbm::get_populations_impl<3>(*s, df, dtype, &s->launches);
     if (!on_device && e == cudaSuccess) e = cudaMemcpyAsync(f, df, bytes, cudaMemcpyDeviceToHost, s->stream);
     if (!on_device) cudaFreeAsync(df, s->stream);
-    cudaError_t e2 = cudaStreamSynchronize(s->stream);
-    if (e == cudaSuccess) e = e2;
-    if (e != cudaSuccess) return cuda_fail(e, "elbm_get_populations");
-    return check_status(s);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(s->stream);
+        return cuda_fail(e, "elbm_get_populations");
+    }
+    return check_status(s, "elbm_get_populations");
 }
 
 int elbm_set_populations(elbm_solver* s, const void* f, int dtype, int on_device)
@@ -612,10 +628,14 @@ static cudaError_t ensure_reduce_scratch(elbm_solver* s)
         s->red_blocks = std::max(1, std::min(8 * s->num_sms, (int)((s->N + 255) / 256)));
         const size_t rows = 2 * (size_t)s->red_blocks;
         e = cudaMallocAsync((void**)&s->partials, sizeof(double) * ELBM_NRED * rows, s->stream);
-        if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->red_out, sizeof(double) * ELBM_NRED, s->stream);
+        if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->red_out, sizeof(double) * (ELBM_NRED + 1), s->stream);
+        if (e == cudaSuccess) e = cudaMallocAsync((void**)&s->red_counter, sizeof(unsigned), s->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(s->red_counter, 0, sizeof(unsigned), s->stream);
         if (e != cudaSuccess) {
-            if (s->partials) cudaFreeAsync(s->partials, s->stream);
+            for (void* ptr : {(void*)s->partials, (void*)s->red_out, (void*)s->red_counter})
+                if (ptr) cudaFreeAsync(ptr, s->stream);
             s->partials = s->red_out = nullptr;
+            s->red_counter = nullptr;
             return e;
         }
         s->bytes += sizeof(double) * ELBM_NRED * (rows + 1);
@@ -637,12 +657,10 @@ int elbm_reduce(elbm_solver* s, double* out)
     }
     if (e != cudaSuccess) return cuda_fail(e, "elbm_reduce scratch");
     e = (s->D == 2) ? elbm::reduce_impl<2>(*s, &s->launches) : elbm::reduce_impl<3>(*s, &s->launches);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->host_red, s->red_out, sizeof(double) * ELBM_NRED, cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e == cudaSuccess) e = fetch_reduction(s);
     if (e != cudaSuccess) return cuda_fail(e, "elbm_reduce");
     std::memcpy(out, s->host_red, sizeof(double) * ELBM_NRED);
-    int rc = check_status(s);
+    const int rc = report_status(s, (int)s->host_red[ELBM_NRED]);
     if (rc != ELBM_OK) return rc;
     if (out[10] > 0.0) return fail(ELBM_ERR_NONFINITE, "%.0f nodes hold non-finite values", out[10]);
     return ELBM_OK;
@@ -665,13 +683,11 @@ int elbm_mode_sums(elbm_solver* s, const double* k, const double* dir, double* o
     if (e != cudaSuccess) return cuda_fail(e, "elbm_mode_sums scratch");
     e = (s->D == 2) ? elbm::mode_sums_impl<2>(*s, k, dir, &s->launches)
                     : elbm::mode_sums_impl<3>(*s, k, dir, &s->launches);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->host_red, s->red_out, sizeof(double) * ELBM_NRED, cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e == cudaSuccess) e = fetch_reduction(s);
     if (e != cudaSuccess) return cuda_fail(e, "elbm_mode_sums");
     out[0] = s->host_red[0];
     out[1] = s->host_red[1];
-    return check_status(s);
+    return report_status(s, (int)s->host_red[ELBM_NRED]);
 }
 
 int elbm_kernel_form(const elbm_solver* s, int* variant)

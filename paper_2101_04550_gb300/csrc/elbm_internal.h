@@ -75,9 +75,10 @@ struct Solver {
     int* status = nullptr;            // device status word
     float* vel = nullptr;             // reduction scratch: the velocity field
     double* partials = nullptr;       // reduction scratch: per-block FP64 partial sums (2 red_blocks rows)
-    double* red_out = nullptr;        // device copy of the ELBM_NRED results
+    double* red_out = nullptr;        // device copy of the ELBM_NRED results and the status word
+    unsigned* red_counter = nullptr;  // blocks done of the running reduction (zero between launches)
     double* factors = nullptr;        // mode projection scratch: a complex factor per node of each axis
-    double host_red[ELBM_NRED] = {};  // host copy of the results
+    double host_red[ELBM_NRED + 1] = {};  // host copy of the results and the status word
     int red_blocks = 0;
     long long steps_done = 0;
     long long launches = 0;
@@ -118,6 +119,10 @@ template <int D> cudaError_t step_bounded_impl(const Solver&, int, long long*);
 template <int D> cudaError_t step_single_impl(const Solver&, void*, long long*);
 template <> cudaError_t step_single_impl<2>(const Solver&, void*, long long*);  // kernels_d2q9.cu
 cudaError_t launch_single_ragged(const Solver& s, const StepParams& p, void* dst);  // single_pass_ragged.cu
+// Several single-pass steps of a small D2Q9 grid in one launch (cluster_d2q9.cuh),
+// in place in s.f: whether s is small enough, and nsteps steps.
+bool small_d2q9(const Solver& s);
+cudaError_t steps_small_d2q9(const Solver& s, int nsteps, long long* launches);
 bool single_tmem_geometry(const Solver& s);
 bool fused_available(const Solver& s);
 cudaError_t step_fused_impl(const Solver& s, int parity, unsigned long long* progress, unsigned long long epoch,

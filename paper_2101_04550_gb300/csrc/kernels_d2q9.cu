@@ -1,5 +1,6 @@
 // Instantiation of the step kernels and their launchers for the D2Q9 lattice.
 #include "step_kernels.cuh"
+#include "cluster_d2q9.cuh"
 #include "single_pass_d2q9.cuh"
 #include "graph_step.cuh"
 #include "batch.cuh"
@@ -12,6 +13,11 @@ template <>
 cudaError_t step_single_impl<2>(const Solver& s, void* dst, long long* launches)
 {
     return step_single_d2q9(s, dst, launches);
+}
+bool small_d2q9(const Solver& s) { return cluster_d2q9_applies(s); }
+cudaError_t steps_small_d2q9(const Solver& s, int nsteps, long long* launches)
+{
+    return steps_cluster_d2q9(s, nsteps, launches);
 }
 template cudaError_t build_step_graph_impl<2>(const Solver&, int, cudaGraphExec_t*, int*);
 template cudaError_t batch_enqueue_impl<2>(int, int, int, int, const void*, int, cudaStream_t, long long*);

@@ -156,3 +156,14 @@ def test_single_pass_repeats_its_bits():
                     if kernel == 3:
                         assert torch.equal(out, got[0])
                 got.append(out.clone())
+
+
+# small D2Q9 grids, several steps a launch in one cluster: one to eight bands of
+# rows, a short last band, several nodes a thread, 16-bit rows; single steps between
+@pytest.mark.parametrize("n", [(3, 3), (64, 64), (33, 5), (100, 37), (17, 129), (500, 18), (1536, 8), (1537, 8)])
+@pytest.mark.parametrize("storage", [elbm.F32, elbm.F32_SHIFT, elbm.F16_SHIFT, elbm.BF16_SHIFT])
+@pytest.mark.parametrize("equilibrium", [0, 1])
+def test_small_d2q9_bitwise(n, storage, equilibrium):
+    kw = dict(stretch=(1.5, 1.0), equilibrium=equilibrium)
+    want = populations(elbm.D2Q9, n, storage, 1, (2, 1, 33), **kw)
+    assert np.array_equal(populations(elbm.D2Q9, n, storage, 3, (2, 1, 33), **kw), want)
