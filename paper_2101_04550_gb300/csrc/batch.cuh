@@ -63,16 +63,23 @@ __global__ void __launch_bounds__(BS) k_batch_anomaly(const BatchMember* __restr
 }
 
 template <int D, int ST, int BS>
-__global__ void __launch_bounds__(BS, 4 * kBlock / BS) k_batch_collide(const BatchMember* __restrict__ table, int count,
-                                                                       int step)
+__global__ void __launch_bounds__(BS, collide_min_blocks<D, ST>() * kBlock / BS)
+    k_batch_collide(const BatchMember* __restrict__ table, int count, int step)
 {
     __shared__ __align__(16) BatchMember m;
-    __shared__ unsigned stage[Lat<D>::Q * BS];
     load_member<BS>(table, count, m);
     const int cell = (blockIdx.x - m.block_begin[BS == 128 ? 0 : 1]) * BS + threadIdx.x;
-    if (cell >= m.p.N) return;
-    if (((m.parity + step) & 1) == 0) collide_staged<D, ST, 0, BS>(m.p, cell, stage + threadIdx.x);
-    else collide_staged<D, ST, 1, BS>(m.p, cell, stage + threadIdx.x);
+    const bool even = ((m.parity + step) & 1) == 0;
+    if constexpr (collide_in_registers<D, ST, false, false, false>()) {
+        if (cell >= m.p.N) return;
+        if (even) collide_node<D, ST, 0>(m.p, cell);
+        else collide_node<D, ST, 1>(m.p, cell);
+    } else {
+        __shared__ unsigned stage[Lat<D>::Q * BS];
+        if (cell >= m.p.N) return;
+        if (even) collide_staged<D, ST, 0, BS>(m.p, cell, stage + threadIdx.x);
+        else collide_staged<D, ST, 1, BS>(m.p, cell, stage + threadIdx.x);
+    }
 }
 
 // Enqueue `nsteps` batched steps on `stream`: for step k, the anomaly pass and

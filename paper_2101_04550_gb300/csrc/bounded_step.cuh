@@ -10,6 +10,23 @@
 
 namespace elbm {
 
+template <int D, int ST, int PAR, bool FX>
+void launch_bounded(const StepParams& p, dim3 grid, cudaStream_t st, long long* launches)
+{
+    if (p.eq_mode == 2) {
+        k_collide<D, ST, PAR, true, true, FX><<<grid, kBlock, 0, st>>>(p);
+    } else {
+        if (p.eq_mode == 0) {
+            k_anomaly<D, ST, PAR, true><<<grid, kBlock, 0, st>>>(p);
+            ++*launches;
+        }
+        k_collide<D, ST, PAR, false, true, FX><<<grid, kBlock, 0, st>>>(p);
+    }
+    ++*launches;
+}
+
+// A force along x alone (or none) takes the lighter force increment, whose registers
+// let the collide kernel gather into registers (collide_in_registers()).
 template <int D>
 cudaError_t step_bounded_impl(const Solver& s, int parity, long long* launches)
 {
@@ -17,18 +34,14 @@ cudaError_t step_bounded_impl(const Solver& s, int parity, long long* launches)
     fill_params(s, p);
     p.parity = parity;
     const dim3 grid((unsigned)((s.N + kBlock - 1) / kBlock));
+    const bool fx = p.g[1] == 0.f && p.g[2] == 0.f;
     ELBM_DISPATCH_STORAGE(s.storage, {
-        if (p.eq_mode == 2) {
-            if (parity == 0) k_collide<D, ST, 0, true, true><<<grid, kBlock, 0, s.stream>>>(p);
-            else k_collide<D, ST, 1, true, true><<<grid, kBlock, 0, s.stream>>>(p);
-        } else if (parity == 0) {
-            if (p.eq_mode == 0) { k_anomaly<D, ST, 0, true><<<grid, kBlock, 0, s.stream>>>(p); ++*launches; }
-            k_collide<D, ST, 0, false, true><<<grid, kBlock, 0, s.stream>>>(p);
-        } else {
-            if (p.eq_mode == 0) { k_anomaly<D, ST, 1, true><<<grid, kBlock, 0, s.stream>>>(p); ++*launches; }
-            k_collide<D, ST, 1, false, true><<<grid, kBlock, 0, s.stream>>>(p);
-        }
-        ++*launches;
+        if (parity == 0)
+            fx ? launch_bounded<D, ST, 0, true>(p, grid, s.stream, launches)
+               : launch_bounded<D, ST, 0, false>(p, grid, s.stream, launches);
+        else
+            fx ? launch_bounded<D, ST, 1, true>(p, grid, s.stream, launches)
+               : launch_bounded<D, ST, 1, false>(p, grid, s.stream, launches);
     });
     return cudaGetLastError();
 }

@@ -49,12 +49,15 @@ __global__ void __launch_bounds__(kBlock) k_anomaly_range(StepParams p, int begi
 }
 
 template <int D, int ST, int PAR>
-__global__ void __launch_bounds__(kBlock, ELBM_COLLIDE_MIN_BLOCKS) k_collide_range(StepParams p, int begin, int end)
+__global__ void __launch_bounds__(kBlock, collide_min_blocks<D, ST>()) k_collide_range(StepParams p, int begin, int end)
 {
-    __shared__ unsigned stage[Lat<D>::Q * kBlock];
     const int cell = begin + blockIdx.x * kBlock + threadIdx.x;
-    if (cell >= end) return;
-    collide_staged<D, ST, PAR>(p, cell, stage + threadIdx.x);
+    if constexpr (collide_in_registers<D, ST, false, false, false>()) {
+        if (cell < end) collide_node<D, ST, PAR>(p, cell);
+    } else {
+        __shared__ unsigned stage[Lat<D>::Q * kBlock];
+        if (cell < end) collide_staged<D, ST, PAR>(p, cell, stage + threadIdx.x);
+    }
 }
 
 // Chunking of the graph-scheduled step: chunks of about 2^18 nodes (a few

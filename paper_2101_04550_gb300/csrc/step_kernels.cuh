@@ -10,11 +10,6 @@ namespace elbm {
 
 constexpr int kBlock = 256;
 
-// Resident blocks per SM the collide kernels are compiled for.
-#ifndef ELBM_COLLIDE_MIN_BLOCKS
-#define ELBM_COLLIDE_MIN_BLOCKS 4
-#endif
-
 #define ELBM_DISPATCH_STORAGE(storage, ...)                              \
     switch (storage) {                                                   \
         case ELBM_F32: { constexpr int ST = ELBM_F32; __VA_ARGS__; } break;             \
@@ -158,7 +153,7 @@ __device__ __forceinline__ void relax_streamed(const StepParams& p, G&& gval, P&
 // warps per SM.  BC: walls (bounce-back slots, and the anomaly's ghost value
 // beyond a wall is the negated value of the wall-adjacent node: Q~_yyy is odd
 // in u_y and u_y = 0 on the wall) and the body force.
-template <int D, int ST, int PAR, int STRIDE = kBlock, bool POLY = false, bool BC = false>
+template <int D, int ST, int PAR, int STRIDE = kBlock, bool POLY = false, bool BC = false, bool FX = false>
 __device__ __forceinline__ void collide_staged(const StepParams& p, int cell, unsigned* col)
 {
     constexpr int Q = Lat<D>::Q;
@@ -196,20 +191,75 @@ __device__ __forceinline__ void collide_staged(const StepParams& p, int cell, un
         if (S::shifted && PAR == 1 && walls && write_bounced(n, i)) gn += bounce_rebase<D>(p, Q - 1 - i);
         S::store(f + slot, S::shifted ? gn : fmaf(p.bw[i], p.rho_ref, gn));
     };
-    relax_streamed<D, POLY, BC>(p, gval, put, drho, j, d);
+    relax_streamed<D, POLY, BC, FX>(p, gval, put, drho, j, d);
 }
 
-// Pass 2 over every node: one node per thread, populations staged in shared
-// memory.  POLY: the conventional second-order equilibrium (no anomaly pass).
-// BC: walls and body force (compiled for one resident block fewer: the force
-// terms need the registers).
-template <int D, int ST, int PAR, bool POLY = false, bool BC = false>
-__global__ void __launch_bounds__(kBlock, BC ? ELBM_COLLIDE_MIN_BLOCKS - 1 : ELBM_COLLIDE_MIN_BLOCKS) k_collide(StepParams p)
+// The same with the populations gathered into registers (27 loads in flight a thread,
+// 24 warps an SM) instead of staged in shared memory by 4-byte cp.async (32 warps).
+// Which one a kernel takes is collide_in_registers().
+template <int D, int ST, int PAR, bool POLY = false, bool BC = false, bool FX = false>
+__device__ __forceinline__ void collide_node(const StepParams& p, int cell)
 {
-    __shared__ unsigned stage[Lat<D>::Q * kBlock];
+    constexpr int Q = Lat<D>::Q;
+    using S = Storage<ST>;
+    const Node n = make_node<D>(p, cell);
+    const bool walls = BC && p.walls_y;
+    float g[Q];
+    gather<D, ST, PAR>(p, n, g, walls);
+    float d[3] = {0.f, 0.f, 0.f};
+    if (p.eq_mode == 0) {
+        const float* q = p.q;
+        d[0] = (q[n.at(1, 0, 0)] - q[n.at(-1, 0, 0)]) * p.inv_2lam[0];
+        const float* qy = q + p.N;
+        const float qyp = (walls && n.yhi) ? -qy[cell] : qy[n.at(0, 1, 0)];
+        const float qym = (walls && n.ylo) ? -qy[cell] : qy[n.at(0, -1, 0)];
+        d[1] = (qyp - qym) * p.inv_2lam[1];
+        if (D == 3) d[2] = (q[2 * p.N + n.at(0, 0, 1)] - q[2 * p.N + n.at(0, 0, -1)]) * p.inv_2lam[2];
+    }
+    auto gval = [&](int i) { return g[i]; };
+    float drho, j[3];
+    moments_of<D>(p, gval, drho, j);
+    typename S::T* f = static_cast<typename S::T*>(p.f);
+    const int cell_o = opaque(cell);
+    auto put = [&](int i, float gn) {
+        const int slot = (PAR == 0) ? (Q - 1 - i) * p.N + cell_o : write_slot<D>(n, p.N, i, PAR, walls);
+        if (S::shifted && PAR == 1 && walls && write_bounced(n, i)) gn += bounce_rebase<D>(p, Q - 1 - i);
+        S::store(f + slot, S::shifted ? gn : fmaf(p.bw[i], p.rho_ref, gn));
+    };
+    relax_streamed<D, POLY, BC, FX>(p, gval, put, drho, j, d);
+}
+
+// Where the register form is the faster one: 16-bit storage, D2Q9, unshifted FP32 and
+// the periodic second-order equilibrium; not with the general body force, whose
+// increment leaves no registers.  us per two-pass step, registers against stage,
+// 135 x 121 x 150: FP16 125 / 136, FP32 161 / 161, FP32-shift 167 / 158; walls and x
+// force FP16 209 / 217, FP32 165 / 178, FP32-shift 200 / 190; second order FP16 76 / 93,
+// FP32-shift 93 / 102 (with walls 136 / 125); D2Q9 2048^2 FP32 95 / 102.
+template <int D, int ST, bool POLY, bool BC, bool FX>
+__host__ __device__ constexpr bool collide_in_registers()
+{
+    if (BC && !FX) return false;
+    return D == 2 || sizeof(typename Storage<ST>::T) == 2 || ST == ELBM_F32 || (POLY && !BC);
+}
+template <int D, int ST, bool POLY = false, bool BC = false, bool FX = false>
+__host__ __device__ constexpr int collide_min_blocks()
+{
+    return collide_in_registers<D, ST, POLY, BC, FX>() || BC ? 3 : 4;
+}
+
+// Pass 2 over every node, one node per thread.  POLY: the conventional second-order
+// equilibrium (no anomaly pass).  BC: walls and body force; FX: the force acts along
+// x alone.
+template <int D, int ST, int PAR, bool POLY = false, bool BC = false, bool FX = false>
+__global__ void __launch_bounds__(kBlock, collide_min_blocks<D, ST, POLY, BC, FX>()) k_collide(StepParams p)
+{
     const int cell = blockIdx.x * kBlock + threadIdx.x;
-    if (cell >= p.N) return;
-    collide_staged<D, ST, PAR, kBlock, POLY, BC>(p, cell, stage + threadIdx.x);
+    if constexpr (collide_in_registers<D, ST, POLY, BC, FX>()) {
+        if (cell < p.N) collide_node<D, ST, PAR, POLY, BC, FX>(p, cell);
+    } else {
+        __shared__ unsigned stage[Lat<D>::Q * kBlock];
+        if (cell < p.N) collide_staged<D, ST, PAR, kBlock, POLY, BC, FX>(p, cell, stage + threadIdx.x);
+    }
 }
 
 template <int D>
