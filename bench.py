@@ -86,7 +86,7 @@ MEASURED_TRAFFIC = {("36d3ed5701ac3c47", "f32s", 0): 5.689e9, ("36d3ed5701ac3c47
 # The sources the step kernels' device code and launch shapes come from (the
 # host-side API, batching and graph code do not change what a kernel moves).
 KERNEL_SOURCES = ("include/elbm.h", "csrc/elbm_internal.h", "csrc/lbm_device.cuh", "csrc/step_kernels.cuh",
-                  "csrc/single_pass.cuh", "csrc/single_pass_tma.cuh", "csrc/single_pass_tmem.cuh",
+                  "csrc/relax_pairs.cuh", "csrc/single_pass.cuh", "csrc/single_pass_tma.cuh", "csrc/single_pass_tmem.cuh",
                   "csrc/tma_maps.cu")
 
 

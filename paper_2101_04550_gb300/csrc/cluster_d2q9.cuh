@@ -16,8 +16,8 @@
 // and values are rounded to the storage type in shared memory as they are in the
 // population array, so the results agree bit for bit.
 //
-// Bound by the two barriers and the dependent chain of a step: 1.85 us at 64 x 64 (one
-// node a thread), 3.1 at 96 x 96.
+// Bound by the two barriers and the dependent chain of a step: 1.55 us at 64 x 64 (one
+// node a thread; 1.85 with its populations and moments read again after the barrier).
 #pragma once
 #include <cooperative_groups.h>
 
@@ -62,26 +62,36 @@ __global__ void __launch_bounds__(kClThreads, 1)
         T* dst = pops + (cur ^ 1) * 9 * plane;
         T* dst_below = cluster.map_shared_rank(dst, below) + (rows_below - 1) * nx;  // its last row
         T* dst_above = cluster.map_shared_rank(dst, above);                          // its first row
-        for (int t = threadIdx.x; t < nodes; t += kClThreads) {
-            float drho, j[3];
-            moments_of<2>(p, [&](int i) { return raw_value<ST>(p, src[i * plane + t], i); }, drho, j);
-            const float inv = 1.0f / (p.rho_ref + drho);
+        // populations and moments of a thread's first node stay in registers over the
+        // barrier; it reads those of further ones again
+        float g0[9], drho0 = 0.f, j0[3] = {0.f, 0.f, 0.f}, inv0 = 1.f;
+        auto load = [&](int t, float* g, float& drho, float* j, float& inv) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g[i] = raw_value<ST>(p, src[i * plane + t], i);
+            moments_of<2>(p, [&](int i) { return g[i]; }, drho, j);
+            inv = 1.0f / (p.rho_ref + drho);
+        };
+        auto publish = [&](int t, const float* j, float inv) {
             qx[t] = anomaly(p, 0, j[0], j[0] * inv);
             const float q = anomaly(p, 1, j[1], j[1] * inv);
             qy[nx + t] = q;
             if (t < nx) qy_below[t] = q;
             if (t >= nodes - nx) qy_above[t - (nodes - nx)] = q;
+        };
+        if (threadIdx.x < nodes) {
+            load(threadIdx.x, g0, drho0, j0, inv0);
+            publish(threadIdx.x, j0, inv0);
+        }
+        for (int t = threadIdx.x + kClThreads; t < nodes; t += kClThreads) {
+            float g[9], drho, j[3], inv;
+            load(t, g, drho, j, inv);
+            publish(t, j, inv);
         }
         cluster.sync();
-        for (int t = threadIdx.x; t < nodes; t += kClThreads) {
+        auto relax_node = [&](int t, const float* g, float drho, const float* j, float inv) {
             const int y = fast_div(t, p.div_nx_m, p.div_nx_s), x = t - y * nx;
             const int xo[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
-            float g[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) g[i] = raw_value<ST>(p, src[i * plane + t], i);
-            auto gval = [&](int i) { return g[i]; };
-            float drho, j[3], d[3] = {0.f, 0.f, 0.f};
-            moments_of<2>(p, gval, drho, j);
+            float d[3] = {0.f, 0.f, 0.f};
             if (p.eq_mode == 0) {
                 d[0] = (qx[t - x + xo[2]] - qx[t - x + xo[0]]) * p.inv_2lam[0];
                 d[1] = (qy[2 * nx + t] - qy[t]) * p.inv_2lam[1];
@@ -91,7 +101,13 @@ __global__ void __launch_bounds__(kClThreads, 1)
             auto put = [&](int i, float gn) {
                 row[cy_of(i) + 1][i * plane + xo[cx_of(i) + 1]] = S::cvt(S::shifted ? gn : fmaf(p.bw[i], p.rho_ref, gn));
             };
-            relax_streamed<2>(p, gval, put, drho, j, d);
+            relax_streamed<2>(p, [&](int i) { return g[i]; }, put, drho, j, d, inv);
+        };
+        if (threadIdx.x < nodes) relax_node(threadIdx.x, g0, drho0, j0, inv0);
+        for (int t = threadIdx.x + kClThreads; t < nodes; t += kClThreads) {
+            float g[9], drho, j[3], inv;
+            load(t, g, drho, j, inv);
+            relax_node(t, g, drho, j, inv);
         }
         cur ^= 1;
         cluster.sync();  // the pushes have landed, the anomaly may be overwritten
@@ -111,7 +127,7 @@ inline size_t cluster_smem(const Solver& s)
 }
 
 // Whether calls of several steps of s take the cluster: the band in shared memory,
-// and at most kClMaxNodes nodes a block.  us per step, cluster against march: 64 x 64 1.9 / 4.1,
+// and at most kClMaxNodes nodes a block.  us per step, cluster against march: 64 x 64 1.6 / 4.1,
 // 96 x 96 (1152 nodes a block) 3.1 / 4.15 FP32 and 2.8 / 4.2 FP16, 128 x 128 (2048)
 // 4.4 / 4.2 and 3.9 / 4.4, 160 x 100 4.3 / 4.2.
 constexpr int kClMaxNodes = 3 * kClThreads;
