@@ -99,8 +99,10 @@ extern "C" {
  *       the anomaly around its tile and reads the populations once.  D3Q27:
  *       TMA-fed with the populations parked in tensor memory when nx is a
  *       multiple of 32 and ny of 16; 32 x 8 TMA tiles when ny is a multiple
- *       of 8; cp.async-staged otherwise.  D2Q9: strips of 126 columns
- *       marching along y, any grid.  Setting it allocates the second array.
+ *       of 8; fed by cp.async otherwise.  D2Q9: strips of 126 columns
+ *       marching along y, any grid; a call of several steps of a small grid
+ *       is one launch of a thread-block cluster.  Setting it allocates the
+ *       second array.
  *   The second-order equilibrium always runs in the two-pass form; walls and
  *   the body force run in form 3 only on the D3Q27 TMEM geometry (nx a
  *   multiple of 32, ny of 16) and in the two-pass form otherwise. */
@@ -228,7 +230,7 @@ int elbm_sync(elbm_solver* s);
  * see there), or
  * ELBM_ERR_ARG for NULL.  For form 3, *variant (if not NULL) receives the
  * single-pass kernel: 1 TMEM (32 x 16 tiles), 2 TMA (32 x 8 tiles),
- * 3 cp.async-staged (D3Q27), 4 the D2Q9 row march; 0 for the other forms.
+ * 3 cp.async-fed (D3Q27), 4 the D2Q9 row march; 0 for the other forms.
  * Host-side query, no CUDA call. */
 int elbm_kernel_form(const elbm_solver* s, int* variant);
 

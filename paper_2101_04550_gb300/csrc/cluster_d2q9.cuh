@@ -131,9 +131,51 @@ inline size_t cluster_smem(const Solver& s)
 // 96 x 96 (1152 nodes a block) 3.1 / 4.15 FP32 and 2.8 / 4.2 FP16, 128 x 128 (2048)
 // 4.4 / 4.2 and 3.9 / 4.4, 160 x 100 4.3 / 4.2.
 constexpr int kClMaxNodes = 3 * kClThreads;
+constexpr size_t kClMaxSmem = 220 * 1024;
+
+// Launch configuration of the cluster of s.
+struct ClusterLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    explicit ClusterLaunch(const Solver& s)
+    {
+        const int band = cluster_band(s);
+        cfg.gridDim = dim3((unsigned)((s.ny + band - 1) / band));
+        cfg.blockDim = dim3(kClThreads);
+        cfg.dynamicSmemBytes = cluster_smem(s);
+        cfg.stream = s.stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cfg.gridDim.x;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
+// Whether the device can hold the cluster (asked once per solver).
+template <int ST>
+bool cluster_fits(const Solver& s)
+{
+    if (s.cluster_ok < 0) {
+        int clusters = 0;
+        ClusterLaunch l(s);
+        cudaError_t e = set_smem_limit_once<k_cluster_d2q9<ST>>((int)kClMaxSmem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_cluster_d2q9<ST>, &l.cfg);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        s.cluster_ok = e == cudaSuccess && clusters > 0 ? 1 : 0;
+    }
+    return s.cluster_ok == 1;
+}
+
 inline bool cluster_d2q9_applies(const Solver& s)
 {
-    return s.D == 2 && (long long)cluster_band(s) * s.nx <= kClMaxNodes && cluster_smem(s) <= 220 * 1024;
+    if (s.D != 2 || (long long)cluster_band(s) * s.nx > kClMaxNodes || cluster_smem(s) > kClMaxSmem) return false;
+    switch (s.storage) {
+        case ELBM_F32: return cluster_fits<ELBM_F32>(s);
+        case ELBM_F32_SHIFT: return cluster_fits<ELBM_F32_SHIFT>(s);
+        case ELBM_F16_SHIFT: return cluster_fits<ELBM_F16_SHIFT>(s);
+        default: return cluster_fits<ELBM_BF16_SHIFT>(s);
+    }
 }
 
 inline cudaError_t steps_cluster_d2q9(const Solver& s, int nsteps, long long* launches)
@@ -141,24 +183,11 @@ inline cudaError_t steps_cluster_d2q9(const Solver& s, int nsteps, long long* la
     StepParams p;
     fill_params(s, p);
     p.parity = 0;
-    const int band = cluster_band(s);
-    const size_t smem = cluster_smem(s);
+    const ClusterLaunch l(s);
     cudaError_t e = cudaSuccess;
     for (int left = nsteps; left > 0 && e == cudaSuccess; left -= kClMaxSteps) {
         ELBM_DISPATCH_STORAGE(s.storage, {
-            e = set_smem_limit_once<k_cluster_d2q9<ST>>(220 * 1024);
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)((s.ny + band - 1) / band));
-            cfg.blockDim = dim3(kClThreads);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = s.stream;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = cfg.gridDim.x;
-            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_cluster_d2q9<ST>, p, band, std::min(left, kClMaxSteps));
+            e = cudaLaunchKernelEx(&l.cfg, k_cluster_d2q9<ST>, p, cluster_band(s), std::min(left, kClMaxSteps));
         });
         if (e == cudaSuccess) ++*launches;
     }

@@ -94,6 +94,7 @@ struct Solver {
     // planes per segment of the D3Q27 single-pass launches with one and with two
     // resident blocks per SM (0: not computed yet; segment_planes())
     mutable int seg_planes[2] = {0, 0};
+    mutable int cluster_ok = -1;      // the D2Q9 cluster fits the device (-1: not asked yet)
 };
 
 // One member of a batch (see batch.cuh).

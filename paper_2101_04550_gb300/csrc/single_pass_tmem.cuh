@@ -24,9 +24,9 @@
 // previous plane covers the next load.  There is no block-wide barrier in the loop.
 //
 // What bounds it: FP32 storage the memory system, with pushes that straddle tile
-// edges (see launch_single_tmem()); 16-bit storage instruction issue, about 750
+// edges (see launch_single_tmem()); 16-bit storage instruction issue, 736
 // instructions a node (824 before the relaxation took the populations in pairs and
-// the pushes one pointer per c_x; FP32 685, before 763), issued on 70 % of the cycles.
+// the pushes one pointer per c_x; FP32 663, before 763), issued on 72 % of the cycles.
 // Every wait is bounded (2 s, or as soon as another thread of the block gave
 // up); a wait that gives up sets ELBM_ERR_TIMEOUT in the status word, and the
 // block winds down: the loader waits, again bounded, for the copies in flight,
