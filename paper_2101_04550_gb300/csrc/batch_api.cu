@@ -30,6 +30,7 @@
 #include <utility>
 #include <vector>
 
+#include "batch_work.h"
 #include "elbm_internal.h"
 
 struct elbm_batch {
@@ -394,30 +395,11 @@ cudaError_t sp_upload_work(elbm_batch* b, const std::vector<elbm_solver*>& flat,
     std::vector<long long> sig{c};
     for (const auto* s : flat) sig.insert(sig.end(), {s->uid, s->nx, s->ny, s->nz});
     if (sig == b->sp_work_sig && b->sp_work_dev) return cudaSuccess;
-    const int seg = kSegCand[c % 3], rows = cfg_tile_rows(c);
-    std::vector<std::vector<int4>> per(flat.size());
-    for (size_t m = 0; m < flat.size(); ++m) {
-        const elbm_solver* s = flat[m];
-        for (int z0 = 0; z0 < s->nz; z0 += seg)
-            for (int y0 = 0; y0 < s->ny; y0 += rows)
-                for (int x0 = 0; x0 < s->nx; x0 += 32)
-                    per[m].push_back(make_int4((int)m, x0, y0, z0 | (std::min(s->nz, z0 + seg) << 16)));
-    }
-    std::vector<int4> work;
-    if (!cfg_interleaved(c)) {
-        for (auto& v : per) work.insert(work.end(), v.begin(), v.end());
-    } else {
-        for (size_t k = 0;; ++k) {
-            bool any = false;
-            for (auto& v : per)
-                if (k < v.size()) {
-                    work.push_back(v[k]);
-                    any = true;
-                }
-            if (!any) break;
-        }
-    }
-    const size_t bytes = work.size() * sizeof(int4);
+    std::vector<elbm::WorkGrid> grids;
+    for (const auto* s : flat) grids.push_back({s->nx, s->ny, s->nz});
+    const std::vector<elbm::WorkItem> work =
+        elbm::work_list(grids, 32, cfg_tile_rows(c), kSegCand[c % 3], cfg_interleaved(c));
+    const size_t bytes = work.size() * sizeof(elbm::WorkItem);
     if (bytes > b->sp_work_cap) {
         cudaError_t e = cudaStreamSynchronize(b->exec_stream);
         if (b->sp_work_dev) cudaFree(b->sp_work_dev);

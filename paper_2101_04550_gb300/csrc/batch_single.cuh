@@ -13,6 +13,7 @@
 // ring anomaly it recomputes, and the anomaly of a node is the same function
 // of its populations wherever it is computed.
 #pragma once
+#include "batch_work.h"
 #include "single_pass_tmem.cuh"
 
 namespace elbm {
@@ -44,15 +45,14 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* map)
 template <int ST>
 constexpr int kBatchBuffers = sizeof(typename Storage<ST>::T) == 4 ? 1 : 2;
 
-// Work item: x = member, y = x0, z = y0, w = z0 | (z1 << 16).
 template <int ST, bool BC, bool FX>
 __global__ void __launch_bounds__(kTmThreads, 1)
-    k_single_pass_tmem_batch(const SpMember* __restrict__ members, const int4* __restrict__ work, int step)
+    k_single_pass_tmem_batch(const SpMember* __restrict__ members, const WorkItem* __restrict__ work, int step)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) StepParams sp;
-    const int4 w = work[blockIdx.x];
-    const SpMember* m = members + w.x;
+    const WorkItem w = work[blockIdx.x];
+    const SpMember* m = members + w.member;
     const int a = (m->phase + step) & 1;
     const unsigned* src = reinterpret_cast<const unsigned*>(&m->params[a]);
     unsigned* dstw = reinterpret_cast<unsigned*>(&sp);
@@ -62,20 +62,20 @@ __global__ void __launch_bounds__(kTmThreads, 1)
         tensormap_acquire(&m->maps16[a][1]);
     }
     __syncthreads();
-    tmem_tile_step<ST, kTileX, kBatchBuffers<ST>, BC, FX>(&m->maps16[a][0], &m->maps16[a][1], sp, m->params[a ^ 1].f, w.y, w.z,
-                                       w.w & 0xffff, w.w >> 16, smem_raw);
+    tmem_tile_step<ST, kTileX, kBatchBuffers<ST>, BC, FX>(&m->maps16[a][0], &m->maps16[a][1], sp, m->params[a ^ 1].f,
+                                                          w.x0, w.y0, w.z0, w.z0 + w.planes, smem_raw);
 }
 
 // The same over 32 x 8 tile columns with the TMA kernel's tile body
 // (periodic, unforced members; two blocks per SM).
 template <int ST>
 __global__ void __launch_bounds__(kTmaThreads, 2)
-    k_single_pass_tma_batch(const SpMember* __restrict__ members, const int4* __restrict__ work, int step)
+    k_single_pass_tma_batch(const SpMember* __restrict__ members, const WorkItem* __restrict__ work, int step)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) StepParams sp;
-    const int4 w = work[blockIdx.x];
-    const SpMember* m = members + w.x;
+    const WorkItem w = work[blockIdx.x];
+    const SpMember* m = members + w.member;
     const int a = (m->phase + step) & 1;
     const unsigned* src = reinterpret_cast<const unsigned*>(&m->params[a]);
     unsigned* dstw = reinterpret_cast<unsigned*>(&sp);
@@ -85,12 +85,12 @@ __global__ void __launch_bounds__(kTmaThreads, 2)
         tensormap_acquire(&m->maps8[a][1]);
     }
     __syncthreads();
-    tma_tile_step<ST>(&m->maps8[a][0], &m->maps8[a][1], sp, m->params[a ^ 1].f, w.y, w.z, w.w & 0xffff, w.w >> 16,
+    tma_tile_step<ST>(&m->maps8[a][0], &m->maps8[a][1], sp, m->params[a ^ 1].f, w.x0, w.y0, w.z0, w.z0 + w.planes,
                       smem_raw);
 }
 
 template <int ST>
-cudaError_t sp_batch_launch_tma(const SpMember* members, const int4* work, int nwork, int nsteps, cudaStream_t st)
+cudaError_t sp_batch_launch_tma(const SpMember* members, const WorkItem* work, int nwork, int nsteps, cudaStream_t st)
 {
     const int smem = TmaLayout<ST>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tma_batch<ST>>(smem);
@@ -102,7 +102,7 @@ cudaError_t sp_batch_launch_tma(const SpMember* members, const int4* work, int n
 }
 
 template <int ST, bool BC, bool FX>
-cudaError_t sp_batch_launch(const SpMember* members, const int4* work, int nwork, int nsteps, cudaStream_t st)
+cudaError_t sp_batch_launch(const SpMember* members, const WorkItem* work, int nwork, int nsteps, cudaStream_t st)
 {
     const int smem = TmemLayout<ST, kTileX, kBatchBuffers<ST>>::bytes;
     cudaError_t e = set_smem_limit_once<k_single_pass_tmem_batch<ST, BC, FX>>(smem);
@@ -159,7 +159,7 @@ cudaError_t sp_batch_enqueue(int storage, int tile_y, bool bc, bool fx, const vo
 {
     if (nwork <= 0 || nsteps <= 0) return cudaSuccess;
     const SpMember* m = static_cast<const SpMember*>(members);
-    const int4* w = static_cast<const int4*>(work);
+    const WorkItem* w = static_cast<const WorkItem*>(work);
     cudaError_t e = cudaSuccess;
     ELBM_DISPATCH_STORAGE(storage, {
         e = tile_y == kTileY ? sp_batch_launch_tma<ST>(m, w, nwork, nsteps, st)

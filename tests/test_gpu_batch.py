@@ -277,3 +277,36 @@ def test_d2q9_single_pass_members_batch_bitwise():
         assert np.array_equal(s.get_populations(), m.get_populations())
     for s in solo + mixed:
         s.close()
+
+
+@pytest.mark.parametrize("n,configs", [((32, 16, 32769), (0, 5, 6)), ((32, 16, 65545), (1, 9)), ((32, 8, 65545), (8,))])
+def test_single_pass_batch_of_long_grids_bitwise(n, configs):
+    """Grids of more than 2^15 and 2^16 planes in the flattened kernels (tiles of
+    16 and of 8 rows), beside a small member: bit for bit the solo states."""
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rho = torch.ones(n[::-1], device="cuda")
+    u = 0.05 * (2.0 * torch.rand((3,) + n[::-1], device="cuda", generator=g) - 1.0)
+
+    def make(k):
+        small = (32, 16, 8)
+        s = elbm.Solver(elbm.D3Q27, n if k == 0 else small, stretch=(1.0, 1.5, 1.0), T=0.42, nu=0.02,
+                        storage=elbm.F16_SHIFT, kernel=3, stream=torch.cuda.current_stream())
+        s.init(rho if k == 0 else rho[:8, :1].expand(8, 16, 32).contiguous(),
+               u if k == 0 else u[:, :8, :1].expand(3, 8, 16, 32).contiguous())
+        return s
+
+    solo, mixed = [make(0), make(1)], [make(0), make(1)]
+    for s in solo:
+        s.step(2 * len(configs))
+    with elbm.Batch(mixed) as b:
+        for c in configs:
+            b.set_config(c)
+            b.step(2)
+    for s, m in zip(solo, mixed):
+        want = torch.empty((27,) + s.shape, device="cuda")
+        got = torch.empty_like(want)
+        s.get_populations(want)
+        m.get_populations(got)
+        assert torch.equal(got, want)
+        s.close()
+        m.close()
