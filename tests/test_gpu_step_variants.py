@@ -167,3 +167,27 @@ def test_small_d2q9_bitwise(n, storage, equilibrium):
     kw = dict(stretch=(1.5, 1.0), equilibrium=equilibrium)
     want = populations(elbm.D2Q9, n, storage, 1, (2, 1, 33), **kw)
     assert np.array_equal(populations(elbm.D2Q9, n, storage, 3, (2, 1, 33), **kw), want)
+
+
+# the reductions' compensated sums over many nodes a thread: 64-bit sums of the same
+# FP32 terms.  A thread's sum is within kFold n 2^-49 of its terms' magnitudes (kFold = 8
+# terms between folds, n terms), the FP64 sums add less than 2^-40.
+@pytest.mark.parametrize("tail", [2.9e-9, 3.1e-9, 3.4e-9])
+def test_sum_of_a_large_term_and_many_small_ones(tail):
+    """A jet in the rows that are every thread's first node, a nearly quiescent
+    field behind it: a thread adds hundreds of terms below half a unit in the
+    last place of its sum."""
+    N = 8192
+    u = torch.zeros((2, N, N), device="cuda")
+    u[0] = tail
+    u[0, :14] = 0.1   # 114688 nodes; the reduction has some 117000 threads
+    with elbm.Solver(elbm.D2Q9, (N, N), storage=elbm.F32_SHIFT, kernel=1, T=0.42, nu=0.02,
+                     stream=torch.cuda.current_stream()) as s:
+        s.init(torch.ones((N, N), device="cuda"), u)
+        red = s.reduce()
+        rho = torch.empty((N, N), device="cuda")
+        s.moments(rho, u)
+        terms = rho * u[0]   # in FP32, as the kernel forms them
+    want, size = float(terms.double().sum()), float(terms.double().abs().sum())
+    n = -(-N * N // 114688)
+    assert abs(red["mom_x"] - want) <= (8 * n * 2.0 ** -49 + 2.0 ** -40) * size
