@@ -191,3 +191,21 @@ def test_sum_of_a_large_term_and_many_small_ones(tail):
     want, size = float(terms.double().sum()), float(terms.double().abs().sum())
     n = -(-N * N // 114688)
     assert abs(red["mom_x"] - want) <= (8 * n * 2.0 ** -49 + 2.0 ** -40) * size
+
+
+# read-outs of one array at odd parity (bounced slots with walls, none without) against
+# the own-location layout of the single pass: the same state, so the same bits
+@pytest.mark.parametrize("lattice,n,walls", [(elbm.D3Q27, (64, 32, 9), False), (elbm.D3Q27, (64, 32, 9), True),
+                                             (elbm.D2Q9, (65, 33), False)])
+@pytest.mark.parametrize("storage", [elbm.F32, elbm.F32_SHIFT, elbm.F16_SHIFT, elbm.BF16_SHIFT])
+def test_read_outs_at_odd_parity(lattice, n, walls, storage):
+    rho, u = field(lattice, n)
+    got = []
+    for kernel in (1, 3):
+        with elbm.Solver(lattice, n, storage=storage, kernel=kernel, T=0.42, nu=0.02, walls_y=walls) as s:
+            s.init(rho, u)
+            s.step(3)
+            r, v = s.moments(dtype=np.float32)
+            got.append((r, v, s.get_populations(), s.reduce(), s.mode_amplitude((0.3, 0.2, 0.1), (0.4, -0.5, 0.6))))
+    for a, b in zip(*got):
+        assert a == b if isinstance(a, (dict, float)) else np.array_equal(a, b)
