@@ -363,6 +363,25 @@ __global__ void __launch_bounds__(kBlock) k_mode_factors(StepParams p, ModeArgs 
     factors[t] = make_double2(cs, sn);
 }
 
+// u . dir of a node, in FP64.
+template <int D, int ST>
+__device__ __forceinline__ double mode_velocity(const StepParams& p, const Node& n, const ModeArgs& m)
+{
+    float g[Lat<D>::Q];
+    gather_any<D, ST>(p, n, g);
+    float drho, j[3];
+    moments<D>(p, g, drho, j);
+    const float inv_r = 1.0f / (p.rho_ref + drho);
+    double us = 0.0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) us += (double)(j[a] * inv_r + 0.5f * p.g[a]) * m.dir[a];
+    return us;
+}
+__device__ __forceinline__ double2 complex_mul(double2 a, double2 b)
+{
+    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
 template <int D, int ST>
 __global__ void __launch_bounds__(kBlock, 4)
     k_mode_sums(const __grid_constant__ StepParams p, ModeArgs m, const double2* factors, int chunks, int ysegs, int items,
@@ -376,23 +395,36 @@ __global__ void __launch_bounds__(kBlock, 4)
         if (x >= p.nx) continue;
         double re = 0.0, im = 0.0;
         for (int y = y0 + warp; y < y1; y += kBlock / 32) {
-            const Node n = make_node_at<D>(p, x, y, z);
-            float g[Lat<D>::Q];
-            gather_any<D, ST>(p, n, g);
-            float drho, j[3];
-            moments<D>(p, g, drho, j);
-            const float inv_r = 1.0f / (p.rho_ref + drho);
-            double us = 0.0;
-#pragma unroll
-            for (int a = 0; a < D; ++a) us += (double)(j[a] * inv_r + 0.5f * p.g[a]) * m.dir[a];
+            const double us = mode_velocity<D, ST>(p, make_node_at<D>(p, x, y, z), m);
             const double2 fy = factors[p.nx + y];
             re = fma(us, fy.x, re);
             im = fma(us, fy.y, im);
         }
-        const double2 fx = factors[x], fz = factors[p.nx + p.ny + z];
-        const double c = fx.x * fz.x - fx.y * fz.y, s = fx.x * fz.y + fx.y * fz.x;
-        acc[0] += re * c - im * s;
-        acc[1] += re * s + im * c;
+        const double2 f = complex_mul(factors[x], factors[p.nx + p.ny + z]);
+        acc[0] += re * f.x - im * f.y;
+        acc[1] += re * f.y + im * f.x;
+    }
+    block_reduce<2>(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
+    finish_reduction(partials, gridDim.x, 2, counter, p.status, out);
+}
+
+// The same for grids whose planes leave most of a block's columns and rows without a
+// node: a thread takes nodes one by one, whichever they are, and multiplies the three
+// factors of each (14 FP64 operations more a node: a call takes 540 us at 256^3, 354 by
+// rows).  mode_sums_impl() chooses.
+template <int D, int ST>
+__global__ void __launch_bounds__(kBlock, 4)
+    k_mode_sums_nodes(const __grid_constant__ StepParams p, ModeArgs m, const double2* factors, double* partials,
+                      unsigned* counter, double* out)
+{
+    double acc[2] = {0.0, 0.0};
+    for (int cell = blockIdx.x * kBlock + threadIdx.x; cell < p.N; cell += gridDim.x * kBlock) {
+        const int z = (D == 3) ? fast_div(cell, p.div_plane_m, p.div_plane_s) : 0, r = cell - z * p.plane;
+        const int y = fast_div(r, p.div_nx_m, p.div_nx_s), x = r - y * p.nx;
+        const double us = mode_velocity<D, ST>(p, make_node_at<D>(p, x, y, z), m);
+        const double2 f = complex_mul(complex_mul(factors[x], factors[p.nx + y]), factors[p.nx + p.ny + z]);
+        acc[0] = fma(us, f.x, acc[0]);
+        acc[1] = fma(us, f.y, acc[1]);
     }
     block_reduce<2>(acc, partials + (size_t)blockIdx.x * ELBM_NRED);
     finish_reduction(partials, gridDim.x, 2, counter, p.status, out);
@@ -410,11 +442,22 @@ cudaError_t mode_sums_impl(const Solver& s, const double* k, const double* dir, 
     }
     double2* factors = reinterpret_cast<double2*>(s.factors);
     const int nf = s.nx + s.ny + s.nz, chunks = (s.nx + 31) / 32, ysegs = (s.ny + kModeRows - 1) / kModeRows;
-    const int items = chunks * ysegs * s.nz, blocks = std::min(items, s.red_blocks);
+    const int items = chunks * ysegs * s.nz;
+    // Node by node where under three in eight of the threads find a node in a plane's
+    // columns and the rows of a block's warps.  us a call, rows against nodes (and a sine and
+    // cosine a node before both), FP32: 3 x 3 x 30000 230 / 45 (79), 8 x 8 x 4096 73 / 45 (79),
+    // 3 x 128 x 512 81 / 44 (70), 128 x 3 x 512 (3/8) 52 / 44 (70), 15 x 30000 (15/32) 53 / 55
+    // (92), 33 x 4000 (1/2) 35 / 41 (59), 20 x 20000 (5/8) 44 / 51 (87).
+    constexpr int kWarps = kBlock / 32;
+    const bool narrow = 8ll * s.nx * s.ny < 3 * 32ll * chunks * ((s.ny + kWarps - 1) / kWarps * kWarps);
     k_mode_factors<D><<<(nf + kBlock - 1) / kBlock, kBlock, 0, s.stream>>>(p, m, factors);
     ELBM_DISPATCH_STORAGE(s.storage, {
-        k_mode_sums<D, ST><<<blocks, kBlock, 0, s.stream>>>(p, m, factors, chunks, ysegs, items, s.partials, s.red_counter,
-                                                                s.red_out);
+        if (narrow)
+            k_mode_sums_nodes<D, ST><<<s.red_blocks, kBlock, 0, s.stream>>>(p, m, factors, s.partials, s.red_counter,
+                                                                            s.red_out);
+        else
+            k_mode_sums<D, ST><<<std::min(items, s.red_blocks), kBlock, 0, s.stream>>>(p, m, factors, chunks, ysegs, items,
+                                                                                      s.partials, s.red_counter, s.red_out);
     });
     *launches += 2;
     return cudaGetLastError();

@@ -209,3 +209,33 @@ def test_read_outs_at_odd_parity(lattice, n, walls, storage):
             got.append((r, v, s.get_populations(), s.reduce(), s.mode_amplitude((0.3, 0.2, 0.1), (0.4, -0.5, 0.6))))
     for a, b in zip(*got):
         assert a == b if isinstance(a, (dict, float)) else np.array_equal(a, b)
+
+
+# the reductions of grids of several nodes a thread (rows in 16-byte pieces and not), and
+# the mode sums node by node on planes smaller than a block's columns and rows
+@pytest.mark.parametrize("n", [(96, 80, 64), (97, 81, 64), (3, 4, 40000), (12, 9, 5000)])
+@pytest.mark.parametrize("steps,walls", [(0, False), (1, True)])
+def test_diagnostics_of_several_nodes_a_thread(n, steps, walls):
+    test_diagnostics_against_the_read_out_fields(elbm.D3Q27, n, steps, walls)
+
+
+def test_diagnostics_count_non_finite_nodes():
+    """A NaN and an infinite population: counted, left out of the extrema, and
+    reported; the sums over them are not finite."""
+    n = (96, 80, 64)
+    rho, u = field(elbm.D3Q27, n)
+    with elbm.Solver(elbm.D3Q27, n, storage=elbm.F32, kernel=1, T=0.42, nu=0.02) as s:
+        s.init(rho, u)
+        f = s.get_populations()
+        f[3, 0, 0, 5] = np.nan
+        f[13, 63, 79, 95] = np.inf
+        s.set_populations(f)
+        red = s.reduce(raise_nonfinite=False)
+        with pytest.raises(elbm.ElbmError) as err:
+            s.reduce()
+        r, v = s.moments(dtype=np.float32)
+    bad = ~np.isfinite(f).all(0)
+    assert err.value.code == -5 and bad.sum() == 2
+    assert red["nonfinite"] == 2 and not np.isfinite(red["mass"])
+    assert red["umax"] == pytest.approx(np.sqrt((v[:, ~bad].astype(np.float64) ** 2).sum(0).max()), rel=1e-6)
+    assert red["fmin"] == pytest.approx(f[:, ~bad].min(), rel=1e-5)
