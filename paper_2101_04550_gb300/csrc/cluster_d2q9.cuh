@@ -126,8 +126,8 @@ inline size_t cluster_smem(const Solver& s)
     return ((2 * band + 2) * 4 + 18 * band * storage_bytes(s.storage)) * s.nx;
 }
 
-// Whether calls of several steps of s take the cluster: the band in shared memory,
-// and at most kClMaxNodes nodes a block.  us per step, cluster against march: 64 x 64 1.6 / 4.1,
+// Grids the cluster takes: the band in shared memory, and at most kClMaxNodes nodes a
+// block.  us per step, cluster against march: 64 x 64 1.6 / 4.1,
 // 96 x 96 (1152 nodes a block) 3.1 / 4.15 FP32 and 2.8 / 4.2 FP16, 128 x 128 (2048)
 // 4.4 / 4.2 and 3.9 / 4.4, 160 x 100 4.3 / 4.2.
 constexpr int kClMaxNodes = 3 * kClThreads;
@@ -167,9 +167,22 @@ bool cluster_fits(const Solver& s)
     return s.cluster_ok == 1;
 }
 
-inline bool cluster_d2q9_applies(const Solver& s)
+// Steps of a call from which the cluster is the faster one: loading and storing the
+// grid costs as much as one to four steps of the march (us a call, cluster against march,
+// FP32: 64 x 64, one node a thread, 2 steps 8.2 / 8.0, 3 steps 8.3 / 12.0; 128 x 64, two,
+// 3 steps 12.3 / 12.3, 5 steps 17.6 / 20.5; 192 x 64, three, 5 steps 22.6 / 20.5, 50 steps
+// 168 / 205; 1536 x 3 5 steps 22.6 / 18.4, 50 steps 174 / 183).
+inline int cluster_min_steps(const Solver& s)
+{
+    const int per_thread = (cluster_band(s) * s.nx + kClThreads - 1) / kClThreads;
+    return per_thread == 1 ? 3 : per_thread == 2 ? 5 : 16;
+}
+
+// Whether a call of nsteps steps of s takes the cluster.
+inline bool cluster_d2q9_applies(const Solver& s, int nsteps)
 {
     if (s.D != 2 || (long long)cluster_band(s) * s.nx > kClMaxNodes || cluster_smem(s) > kClMaxSmem) return false;
+    if (nsteps < cluster_min_steps(s)) return false;
     switch (s.storage) {
         case ELBM_F32: return cluster_fits<ELBM_F32>(s);
         case ELBM_F32_SHIFT: return cluster_fits<ELBM_F32_SHIFT>(s);

@@ -483,7 +483,7 @@ int elbm_step(elbm_solver* s, int n)
     cudaError_t e = cudaSuccess;
     int left = n;
     while (left > 0 && e == cudaSuccess) {
-        if (kernel == 3 && s->parity == 0 && s->f2 && left > 1 && elbm::small_d2q9(*s)) {
+        if (kernel == 3 && s->parity == 0 && s->f2 && elbm::small_d2q9(*s, left)) {
             // a small D2Q9 grid: every step of the call in one launch, the state stays in f
             e = elbm::steps_small_d2q9(*s, left, &s->launches);
             left = 0;

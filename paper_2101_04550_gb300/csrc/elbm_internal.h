@@ -121,8 +121,9 @@ template <int D> cudaError_t step_single_impl(const Solver&, void*, long long*);
 template <> cudaError_t step_single_impl<2>(const Solver&, void*, long long*);  // kernels_d2q9.cu
 cudaError_t launch_single_ragged(const Solver& s, const StepParams& p, void* dst);  // single_pass_ragged.cu
 // Several single-pass steps of a small D2Q9 grid in one launch (cluster_d2q9.cuh),
-// in place in s.f: whether s is small enough, and nsteps steps.
-bool small_d2q9(const Solver& s);
+// in place in s.f: whether s is small enough and nsteps make it worth while, and
+// nsteps steps.
+bool small_d2q9(const Solver& s, int nsteps);
 cudaError_t steps_small_d2q9(const Solver& s, int nsteps, long long* launches);
 bool single_tmem_geometry(const Solver& s);
 bool fused_available(const Solver& s);

@@ -14,7 +14,7 @@ cudaError_t step_single_impl<2>(const Solver& s, void* dst, long long* launches)
 {
     return step_single_d2q9(s, dst, launches);
 }
-bool small_d2q9(const Solver& s) { return cluster_d2q9_applies(s); }
+bool small_d2q9(const Solver& s, int nsteps) { return cluster_d2q9_applies(s, nsteps); }
 cudaError_t steps_small_d2q9(const Solver& s, int nsteps, long long* launches)
 {
     return steps_cluster_d2q9(s, nsteps, launches);

@@ -239,3 +239,19 @@ def test_diagnostics_count_non_finite_nodes():
     assert red["nonfinite"] == 2 and not np.isfinite(red["mass"])
     assert red["umax"] == pytest.approx(np.sqrt((v[:, ~bad].astype(np.float64) ** 2).sum(0).max()), rel=1e-6)
     assert red["fmin"] == pytest.approx(f[:, ~bad].min(), rel=1e-5)
+
+
+# which calls the cluster takes, by their launches: one to three nodes a thread, the
+# fewest steps of each and one less, more steps than one launch takes, a grid too large
+@pytest.mark.parametrize("n,steps,launches", [((64, 64), 2, 2), ((64, 64), 3, 1), ((128, 64), 4, 4), ((128, 64), 5, 1),
+                                              ((192, 64), 15, 15), ((192, 64), 16, 1), ((33, 5), 4099, 2),
+                                              ((1537, 8), 33, 33)])
+def test_small_d2q9_calls(n, steps, launches):
+    rho, u = field(elbm.D2Q9, n)
+    with elbm.Solver(elbm.D2Q9, n, kernel=3, T=0.42, nu=0.02, stream=torch.cuda.current_stream()) as s:
+        s.init(rho, u)
+        before = s.launches
+        s.step(steps)
+        assert s.launches - before == launches
+        got = s.get_populations()
+    assert np.array_equal(got, populations(elbm.D2Q9, n, elbm.F32, 1, (steps,)).astype(np.float64))
