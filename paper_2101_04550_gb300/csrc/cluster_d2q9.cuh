@@ -21,7 +21,7 @@
 #pragma once
 #include <cooperative_groups.h>
 
-#include "single_pass.cuh"
+#include "single_pass_d2q9.cuh"
 
 namespace elbm {
 
@@ -168,14 +168,20 @@ bool cluster_fits(const Solver& s)
 }
 
 // Steps of a call from which the cluster is the faster one: loading and storing the
-// grid costs as much as one to four steps of the march (us a call, cluster against march,
-// FP32: 64 x 64, one node a thread, 2 steps 8.2 / 8.0, 3 steps 8.3 / 12.0; 128 x 64, two,
-// 3 steps 12.3 / 12.3, 5 steps 17.6 / 20.5; 192 x 64, three, 5 steps 22.6 / 20.5, 50 steps
-// 168 / 205; 1536 x 3 5 steps 22.6 / 18.4, 50 steps 174 / 183).
+// grid costs as much as one to four steps of the march, more where three rows leave it
+// three blocks, less where the march's blocks do not find an SM each.  us a call, cluster
+// against march, FP32 (FP16): 64 x 64, one node a thread, 2 steps 8.2 / 8.0 (6.4 / 8.2);
+// 512 x 3 2 steps 8.2 / 7.2, 3 steps 10.3 / 10.8; 128 x 64, two nodes, 3 steps 12.3 / 12.3,
+// 5 steps 17.6 / 20.5; 192 x 64, three nodes, 5 steps 22.6 / 20.5 (20.5 / 21.8), 50 steps 168 /
+// 205; 1536 x 3 5 steps 22.6 / 18.4, 50 steps 174 / 183; 12 x 1000, 250 blocks of the march,
+// 2 steps 12.3 / 13.1.
 inline int cluster_min_steps(const Solver& s)
 {
-    const int per_thread = (cluster_band(s) * s.nx + kClThreads - 1) / kClThreads;
-    return per_thread == 1 ? 3 : per_thread == 2 ? 5 : 16;
+    const int nodes = cluster_band(s) * s.nx, seg = d2q9_segment_rows(s);
+    const int march_blocks = (s.nx + kD2Cols - 1) / kD2Cols * ((s.ny + seg - 1) / seg);
+    const bool many_rows = s.ny >= kClBlocks;
+    if (march_blocks > s.num_sms || (nodes <= kClThreads && many_rows)) return 2;
+    return nodes <= kClThreads ? 3 : nodes <= 2 * kClThreads ? 5 : many_rows ? 8 : 16;
 }
 
 // Whether a call of nsteps steps of s takes the cluster.

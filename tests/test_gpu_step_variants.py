@@ -242,10 +242,12 @@ def test_diagnostics_count_non_finite_nodes():
 
 
 # which calls the cluster takes, by their launches: one to three nodes a thread, the
-# fewest steps of each and one less, more steps than one launch takes, a grid too large
-@pytest.mark.parametrize("n,steps,launches", [((64, 64), 2, 2), ((64, 64), 3, 1), ((128, 64), 4, 4), ((128, 64), 5, 1),
-                                              ((192, 64), 15, 15), ((192, 64), 16, 1), ((33, 5), 4099, 2),
-                                              ((1537, 8), 33, 33)])
+# fewest steps of each and one less, three blocks and eight, more of the march's blocks
+# than SMs, more steps than one launch takes, a grid too large
+@pytest.mark.parametrize("n,steps,launches", [((64, 64), 1, 1), ((64, 64), 2, 1), ((512, 3), 2, 2), ((512, 3), 3, 1),
+                                              ((128, 64), 4, 4), ((128, 64), 5, 1), ((192, 64), 7, 7),
+                                              ((192, 64), 8, 1), ((1536, 3), 15, 15), ((1536, 3), 16, 1),
+                                              ((12, 1000), 2, 1), ((33, 5), 4099, 2), ((1537, 8), 33, 33)])
 def test_small_d2q9_calls(n, steps, launches):
     rho, u = field(elbm.D2Q9, n)
     with elbm.Solver(elbm.D2Q9, n, kernel=3, T=0.42, nu=0.02, stream=torch.cuda.current_stream()) as s:
