@@ -2,9 +2,12 @@
 // stick out of the grid, loaded by cp.async (tmem_tile_step with PB != 0).  Taken
 // where the TMA-fed kernels do not apply.
 //
-// Bound as the TMA-fed kernel is, plus the idle nodes of tiles that stick out and the
-// loading warps' copies: 180 x 120 x 100 FP32 125 us per step, floor 69; the cp.async-staged
-// kernel with block-wide barriers on 32 x 8 tiles that it replaces took 217.
+// Bound as the TMA-fed kernel is, plus the idle nodes of tiles that stick out.  us per
+// step, one launch per step of the cp.async-staged kernel with block-wide barriers that it
+// replaces against this one: 180 x 120 x 100 FP32-shift 223 / 108, FP16 (rows on 8 bytes)
+// 179 / 122; 161^3 507 / 313 and 416 / 271; 33 x 200 x 100 98 / 70 and 84 / 66; 3^3 15.4 /
+// 8.4.  (With a loop per row in the copies and the ring rows all on one warp, the copies'
+// latency bounded the 4-byte forms: 161^3 750 and 662, 33 x 200 x 100 192 and 167.)
 #include "single_pass_tmem.cuh"
 
 namespace elbm {

@@ -149,7 +149,8 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
             mbar_init(empty_t(b), kTmConsumers);
         }
         for (int r = 0; r < 2; ++r) {
-            mbar_init(full_r(r), (PB == 0 ? 1 : 0) + 32);  // loader lane 0 (expect_tx) + the cp.async arrivals of its 32 lanes
+            // lane 0's expect_tx and the cp.async arrivals of the loading warp, or of the four
+            mbar_init(full_r(r), PB == 0 ? 1 + 32 : 128);
             mbar_init(empty_r(r), 32 * L::ring_warps);
         }
         for (int s = 0; s < kTmaQSlots; ++s) mbar_init(qready(s), kTmConsumers + 32 * L::ring_warps);
@@ -224,7 +225,7 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
         const int cxl = wrapi(x0 - 1, p.nx), cxr = wrapi(x0 + w, p.nx);
         auto load_columns = [&](int zk, int r) {
             unsigned* cols = reinterpret_cast<unsigned*>(base + L::off_cols + r * L::cols_bytes);
-            for (int c = lane; c < 27 * L::ncol; c += 32) {
+            for (int c = PB == 0 ? lane : (int)threadIdx.x - kTmConsumers; c < 27 * L::ncol; c += PB == 0 ? 32 : 128) {
                 const int i = c / L::ncol, kk = c % L::ncol, y = PB == 0 ? kk & (TY - 1) : min(kk & (TY - 1), h - 1);
                 const int idx = i * p.N + zk * p.plane + (y0 + y) * p.nx + (kk < TY ? cxl : cxr);
                 cp_async4(cols + c, stage_src<ST>(p, idx));
@@ -233,49 +234,68 @@ __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const
         };
         int issued = 0;
         if constexpr (PB != 0) {
-            const T* f = static_cast<const T*>(p.f);
-            // rows [0, rows) of w elements, row r of population i starting at element
-            // i N + first + r nx, into dst rows of RS elements (one population)
-            auto copy_rows = [&](T* to, int i, int first, int rows) {
-                const int from = i * p.N + first;
+            // A row goes over in pieces of PB bytes, 16-bit rows on 4-byte pieces in the words
+            // that hold them: lane l takes pieces l, l + 32, ... of the tile's rows of a
+            // population and of its two ring rows, warp q populations q, q + 4, ...  Where a
+            // piece lies is the same in every plane and population, so it is worked out once,
+            // and the copies of a population are independent instructions.
+            constexpr int NPR = PB == 16 ? TX * L::es / 16 : L::es == 4 ? TX : TX / 2 + 1;  // pieces of a row
+            constexpr int EP = PB == 16 ? 16 / L::es : 1;                                   // elements of a piece
+            constexpr int NT_TILE = (TY * NPR + 31) / 32, NT_RING = (2 * NPR + 31) / 32;
+            // first element of the piece (words: of its row) in a plane, or -1 where the
+            // grid has none; its byte among the population's rows in the buffer
+            struct Piece {
+                int from, to;
+            };
+            auto piece = [&](int c, int row, bool any, int stride) {
+                const int x = c % NPR * EP;
+                return Piece{any && (L::words || x < w) ? row * p.nx + x0 + (L::words ? 0 : x) : -1,
+                             c / NPR * stride + c % NPR * PB};
+            };
+            Piece tile_piece[NT_TILE], ring_piece[NT_RING];
+#pragma unroll
+            for (int q = 0; q < NT_TILE; ++q) {
+                const int c = lane + 32 * q;
+                tile_piece[q] = piece(c, y0 + c / NPR, c / NPR < h, RS * L::es);
+            }
+#pragma unroll
+            for (int q = 0; q < NT_RING; ++q) {
+                const int c = lane + 32 * q;
+                ring_piece[q] = piece(c, c / NPR ? yhi : ylo, c / NPR < 2, L::row_stride);
+            }
+            // piece c of a row of the population that starts at element i N + plane
+            auto copy = [&](unsigned char* to, const Piece& q, int c, int start) {
                 if constexpr (PB == 16) {
-                    constexpr int E = 16 / L::es, PPR = TX / E;
-                    for (int c = lane; c < rows * PPR; c += 32) {
-                        const int y = c / PPR, x = c % PPR * E;
-                        if (x < w) cp_async16(to + y * RS + x, f + from + y * p.nx + x);
-                    }
+                    if (q.from >= 0) cp_async16(to + q.to, static_cast<const T*>(p.f) + start + q.from);
                 } else if constexpr (L::es == 4) {
-                    for (int c = lane; c < rows * TX; c += 32) {
-                        const int y = c / TX, x = c % TX;
-                        if (x < w) cp_async4(reinterpret_cast<unsigned*>(to + y * RS + x), f + from + y * p.nx + x);
-                    }
+                    if (q.from >= 0)
+                        cp_async4(reinterpret_cast<unsigned*>(to + q.to), static_cast<const T*>(p.f) + start + q.from);
                 } else {
-                    constexpr int NW = TX / 2 + 1;  // words that can hold a row
-                    for (int c = lane; c < rows * NW; c += 32) {
-                        const int y = c / NW, j = c % NW, at = from + y * p.nx;
-                        if (j < ((at & 1) + w + 1) >> 1)
-                            cp_async4(reinterpret_cast<unsigned*>(to + y * RS) + j,
-                                      static_cast<const unsigned*>(p.f) + (at >> 1) + j);
-                    }
+                    const int at = start + q.from, j = c % NPR;
+                    if (q.from >= 0 && j < ((at & 1) + w + 1) >> 1)
+                        cp_async4(reinterpret_cast<unsigned*>(to + q.to), static_cast<const unsigned*>(p.f) + (at >> 1) + j);
                 }
             };
             for (int k = 0; k < K; ++k) {
                 const int b = k % L::ntile, r = k & 1, zk = plane_of(k);
                 bool ok = true;
                 if (k >= L::ntile) ok = wait(empty_t(b), ((k / L::ntile) - 1) & 1);
-                if (ok && warp == kLoader && k >= 2) ok = wait(empty_r(r), ((k / 2) - 1) & 1);
+                if (ok && k >= 2) ok = wait(empty_r(r), ((k / 2) - 1) & 1);
                 if (!__all_sync(0xffffffffu, ok)) break;
-                T* tile = reinterpret_cast<T*>(base + L::off_tile + b * L::tile_bytes);
-                for (int i = warp - kLoader; i < 27; i += 4) copy_rows(tile + i * TY * RS, i, zk * p.plane + y0 * p.nx + x0, h);
+                for (int i = warp - kLoader; i < 27; i += 4) {
+                    unsigned char* to = base + L::off_tile + b * L::tile_bytes + i * TY * RS * L::es;
+#pragma unroll
+                    for (int q = 0; q < NT_TILE; ++q) copy(to, tile_piece[q], lane + 32 * q, i * p.N + zk * p.plane);
+                }
                 cp_async_mbar_arrive(full_t(b));
                 issued = k + 1;
-                if (warp == kLoader) {
-                    for (int side = 0; side < 2; ++side) {
-                        T* row = reinterpret_cast<T*>(base + L::off_rows + (2 * r + side) * L::row_stride);
-                        for (int i = 0; i < 27; ++i) copy_rows(row + i * RS, i, zk * p.plane + (side ? yhi : ylo) * p.nx + x0, 1);
-                    }
-                    load_columns(zk, r);
-                } else if (k > 0) {  // the ring of the plane before, while this one is on its way
+                for (int i = warp - kLoader; i < 27; i += 4) {
+                    unsigned char* to = base + L::off_rows + 2 * r * L::row_stride + i * RS * L::es;
+#pragma unroll
+                    for (int q = 0; q < NT_RING; ++q) copy(to, ring_piece[q], lane + 32 * q, i * p.N + zk * p.plane);
+                }
+                load_columns(zk, r);
+                if (warp != kLoader && k > 0) {  // the ring of the plane before, while this one is on its way
                     if (!__all_sync(0xffffffffu, wait(full_r(r ^ 1), ((k - 1) / 2) & 1))) break;
                     ring_plane(k - 1);
                 }
