@@ -26,40 +26,46 @@ constexpr int kHalo = 2 * kTileX + 2 * kTileY;
 // relaxes, so long segments re-read little and short ones fill the GPU.  The
 // depth (up to 64) is the one whose schedule ends first when the blocks, in
 // launch order, take the next free of `slots` resident places and a segment
-// of n planes costs n + 2.5: a march is a serial chain of planes (2.0 us each
-// for a 32 x 16 TMEM tile alone on its SM, 2.9 us under full memory traffic)
-// plus the block's start-up.  Measured with that kernel, us per step against
-// the fixed 32 planes used before: 32^3 7.1 (depth 1) against 72.5, 64^3 14.8
-// (4) against 76.2; FP16 storage 96^3 31.0 (12) against 75.9, 128^3 70.6 (29)
-// against 78.4, 160^3 125.5 (54) against 149.6; 256^3 FP32 670.4 (37) against
-// 677.2, FP16 496-500 against 512.
-inline int segment_planes(long long columns, int nz, int slots)
+// of n planes costs n + 2.5: a march is a serial chain of planes plus the block's
+// start-up.  us per step of the TMEM kernel against fixed 32 planes: FP32-shift 64^3
+// 13.4 / 68.8, 96^3 42 / 80, 128^3 84 / 87, 160^3 168 / 183, 192^3 268 / 272, 256^3 621 / 627;
+// FP16 96^3 29 / 68, 128^3 61 / 67, 160^3 121 / 139, 256^3 442 / 450.
+// keep: a depth that stays unless another ends 5 % earlier (0: none).
+inline int segment_planes(long long columns, int nz, int slots, int keep = 0)
 {
-    int best = 1;
-    long long best_end = -1;
-    for (int seg = nz < 64 ? nz : 64; seg >= 1; --seg) {  // costs in half planes
+    auto schedule_end = [&](int seg) {  // in half planes
         const long long nseg = (nz + seg - 1) / seg, len = 2 * seg + 5, last = 2 * (nz - (nseg - 1) * seg) + 5;
         // the full segments launch first, then one last segment per column
         const long long full = (nseg - 1) * columns, rem = full % slots, t0 = (full / slots) * len;
         long long end = t0 + std::max(rem ? len : 0, (columns + slots - 1) / slots * last);
         while ((slots - rem) * ((end - t0) / last) + rem * (end - t0 >= len ? (end - t0 - len) / last : 0) < columns)
             ++end;
+        return end;
+    };
+    int best = 1;
+    long long best_end = -1;
+    for (int seg = nz < 64 ? nz : 64; seg >= 1; --seg) {
+        const long long end = schedule_end(seg);
         if (best_end < 0 || end < best_end) {
             best = seg;
             best_end = end;
         }
     }
-    return best;
+    return keep > 0 && keep <= nz && schedule_end(keep) * 95 <= best_end * 100 ? keep : best;
 }
 
 // ... of a launch over solver s in tiles of tile_x x tile_y columns, per_sm blocks
-// resident on an SM (kept in the solver: the grid and its tiles do not change).
+// resident on an SM (kept in the solver: the grid and its tiles do not change).  Two
+// blocks share an SM's memory traffic, which the schedule does not see: 192 x 200 x 192
+// FP32-shift in 32 x 8 tiles takes 457 us with its 48 planes, 427 with 32 (2 % apart in
+// the schedule), while 160 x 168 x 160 gains 3 % (schedule 7 %) and 96 x 104 x 96 16 %
+// (55 %), so there 32 planes stay unless the schedule ends 5 % earlier.
 inline int solver_segment_planes(const Solver& s, int tile_x, int tile_y, int per_sm)
 {
     int& seg = s.seg_planes[per_sm == 1 ? 0 : 1];
     if (seg == 0)
         seg = segment_planes((long long)((s.nx + tile_x - 1) / tile_x) * ((s.ny + tile_y - 1) / tile_y), s.nz,
-                             per_sm * (s.num_sms > 0 ? s.num_sms : 152));
+                             per_sm * (s.num_sms > 0 ? s.num_sms : 152), per_sm == 1 ? 0 : 32);
     return seg;
 }
 
