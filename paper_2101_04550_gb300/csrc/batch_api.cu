@@ -53,7 +53,9 @@ struct elbm_batch {
     struct MemberGraph {               // form 3: one member's n-step sequence
         long long uid = 0;             // the member's solver (uid, never reused)
         int nsteps = 0;
-        const void* f = nullptr;       // its current array when captured
+        long long revision = 0;        // of its parameters, which the graph's kernels hold
+        const void* f = nullptr;       // its arrays when captured, the current one first
+        const void* f2 = nullptr;
         cudaGraphExec_t exec = nullptr;
         long long launches = 0;
     };
@@ -207,7 +209,7 @@ cudaError_t member_graph(elbm_batch* b, elbm_solver* s, int nsteps, cudaStream_t
                          long long* launches)
 {
     for (const auto& g : b->member_graphs)
-        if (g.uid == s->uid && g.nsteps == nsteps && g.f == s->f) {
+        if (g.uid == s->uid && g.revision == s->revision && g.nsteps == nsteps && g.f == s->f && g.f2 == s->f2) {
             *exec = g.exec;
             *launches = g.launches;
             return cudaSuccess;
@@ -218,8 +220,10 @@ cudaError_t member_graph(elbm_batch* b, elbm_solver* s, int nsteps, cudaStream_t
     seq.stream = ps;
     elbm_batch::MemberGraph g;
     g.uid = s->uid;
+    g.revision = s->revision;
     g.nsteps = nsteps;
     g.f = s->f;
+    g.f2 = s->f2;
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(ps, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;

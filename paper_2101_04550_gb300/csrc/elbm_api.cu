@@ -336,6 +336,7 @@ int elbm_set_option(elbm_solver* s, int key, double value)
 {
     if (!s) return fail(ELBM_ERR_ARG, "solver is NULL");
     drop_graphs(s);
+    ++s->revision;
     switch (key) {
         case ELBM_OPT_EQUILIBRIUM:
             if (value != 0.0 && value != 1.0 && value != 2.0) return fail(ELBM_ERR_ARG, "equilibrium must be 0, 1 or 2");
@@ -453,7 +454,9 @@ int elbm_init(elbm_solver* s, const void* rho, const void* u, int dtype, int on_
                 const double U0 = s->host_red[1 + a] / s->host_red[0];
                 float tri[3];
                 double ueff;
-                s->u_ref[a] = (std::isfinite(U0) && elbm::base_triplet(s->T, s->lam[a], U0, tri, &ueff)) ? U0 : 0.0;
+                const double ref = (std::isfinite(U0) && elbm::base_triplet(s->T, s->lam[a], U0, tri, &ueff)) ? U0 : 0.0;
+                if (s->u_ref[a] != ref) ++s->revision;
+                s->u_ref[a] = ref;
             }
         }
     }

@@ -84,6 +84,7 @@ struct Solver {
     long long launches = 0;
     size_t bytes = 0;
     long long uid = 0;                // unique per solver of the process (never reused)
+    long long revision = 0;           // counts the changes of what fill_params() reads
     // tensor maps of the TMA-fed single-pass kernels, cached per population
     // array and tile shape (tma_maps.cu); a map depends only on the array's
     // address and the grid, so a cached one stays valid for that address

@@ -310,3 +310,58 @@ def test_single_pass_batch_of_long_grids_bitwise(n, configs):
         assert torch.equal(got, want)
         s.close()
         m.close()
+
+
+def _advected(n, speed):
+    rho, u = _fields(n, 3, 3)
+    u[0] += speed
+    return rho, u
+
+
+@pytest.mark.parametrize("config", [0, elbm.BATCH_CONFIGS - 1])
+def test_single_pass_batch_follows_its_members_parameters(config):
+    """A member's equilibrium, body force and automatic storage baseline change
+    between calls of the batch: bit for bit the solo states."""
+    n = (64, 32, 16)
+
+    def make():
+        s = elbm.Solver(elbm.D3Q27, n, stretch=(1.0, 1.5, 1.0), T=0.42, nu=0.02, storage=elbm.F16_SHIFT, kernel=3,
+                        u_ref="mean", stream=torch.cuda.current_stream())
+        s.init(*_advected(n, 0.02))
+        return s
+
+    changes = [lambda s: None, lambda s: s.set_option(elbm.OPT_EQUILIBRIUM, 1),
+               lambda s: s.set_option(elbm.OPT_FORCE_X, 1e-4), lambda s: s.init(*_advected(n, 0.1))]
+    solo, member = make(), make()
+    with elbm.Batch([member]) as b:
+        b.set_config(config)
+        for change in changes:
+            change(solo)
+            change(member)
+            solo.step(4)
+            b.step(4)
+            assert np.array_equal(member.get_populations(), solo.get_populations())
+    solo.close()
+    member.close()
+
+
+def test_single_pass_batch_member_with_new_arrays():
+    """A member gives its second array back and takes another one between calls
+    (the kernel form goes to two-pass and back): its cached graphs do not write
+    to the old one, which another solver may own by then."""
+    n = (64, 32, 16)
+    spec = (n, (1.0, 1.5, 1.0), 0.42, 0.02)
+    solo, member = _make_sp(spec, elbm.F32_SHIFT, 5), _make_sp(spec, elbm.F32_SHIFT, 5)
+    with elbm.Batch([member]) as b:
+        b.set_config(elbm.BATCH_CONFIGS - 1)
+        b.step(4)
+        member.set_option(elbm.OPT_KERNEL, 1)
+        other = _make_sp(spec, elbm.F32_SHIFT, 6)
+        before = other.get_populations()
+        member.set_option(elbm.OPT_KERNEL, 3)
+        b.step(4)
+        solo.step(8)
+        assert np.array_equal(member.get_populations(), solo.get_populations())
+        assert np.array_equal(other.get_populations(), before)
+    for s in (solo, member, other):
+        s.close()
