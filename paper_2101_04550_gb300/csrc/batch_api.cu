@@ -533,16 +533,15 @@ int step_single_form(elbm_batch* b, int nsteps)
     int c = kSpGraphs;
     if (any_flat) {
         const long long key = sp_key(b, b->members);
-        SpTuning* t = nullptr;
-        {
-            std::lock_guard<std::mutex> lock(g_tune_lock);
-            t = &g_sp_tuning[key];  // map nodes stay where they are
-        }
+        // the tuning record is shared with the batches of other threads: one at a time
+        // reads it or goes on with the tuning
+        std::lock_guard<std::mutex> lock(g_tune_lock);
+        SpTuning& t = g_sp_tuning[key];
         // the tuning steps are real steps of every member (an even number, so
         // each state ends in the array it started in)
-        if (t->chosen < 0 && b->sp_pinned < 0) e = sp_tune(b, *t, &left);
+        if (t.chosen < 0 && b->sp_pinned < 0) e = sp_tune(b, t, &left);
         // while still tuning: TMEM tiles, 32-plane segments, member-major
-        c = b->sp_pinned >= 0 ? b->sp_pinned : t->chosen >= 0 ? t->chosen : 0;
+        c = b->sp_pinned >= 0 ? b->sp_pinned : t.chosen >= 0 ? t.chosen : 0;
         b->sp_key = key;
     }
     b->sp_config = c;

@@ -365,3 +365,33 @@ def test_single_pass_batch_member_with_new_arrays():
         assert np.array_equal(other.get_populations(), before)
     for s in (solo, member, other):
         s.close()
+
+
+def test_batches_of_several_threads_tune_together():
+    """Batches of one tuning key stepped by four threads, each on a stream of its
+    own, while the key is still being tuned: bit for bit the solo state."""
+    import threading
+
+    spec = ((96, 32, 41), (1.0, 1.5, 1.0), 0.42, 0.02)
+    want = _make_sp(spec, elbm.BF16_SHIFT, 8)
+    want.step(30)
+    want = want.get_populations()
+    got = {}
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            s = _make_sp(spec, elbm.BF16_SHIFT, 8)
+            with elbm.Batch([s]) as b:
+                for _ in range(10):
+                    b.step(3)
+            got[k] = s.get_populations()
+            s.close()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert len(got) == 4
+    for f in got.values():
+        assert np.array_equal(f, want)
