@@ -101,7 +101,8 @@ extern "C" {
  *       multiple of 32 and ny of 16; 32 x 8 TMA tiles when ny is a multiple
  *       of 8; fed by cp.async otherwise.  D2Q9: strips of 126 columns
  *       marching along y, any grid; a call of several steps of a small grid
- *       is one launch of a thread-block cluster.  Setting it allocates the
+ *       (from two to sixteen steps on, by its size) is one launch of a
+ *       thread-block cluster.  Setting it allocates the
  *       second array.
  *   The second-order equilibrium always runs in the two-pass form; walls and
  *   the body force run in form 3 only on the D3Q27 TMEM geometry (nx a
@@ -229,8 +230,9 @@ int elbm_sync(elbm_solver* s);
  * 3 single pass, 4 fused in place (ELBM_OPT_KERNEL and the grid decide it;
  * see there), or
  * ELBM_ERR_ARG for NULL.  For form 3, *variant (if not NULL) receives the
- * single-pass kernel: 1 TMEM (32 x 16 tiles), 2 TMA (32 x 8 tiles),
- * 3 cp.async-fed (D3Q27), 4 the D2Q9 row march; 0 for the other forms.
+ * single-pass kernel: 1 TMEM (64 x 8 or 32 x 16 tiles), 2 TMA (32 x 8
+ * tiles), 3 cp.async-fed (D3Q27), 4 D2Q9 (the row march, and the cluster
+ * for calls of several steps of a small grid); 0 for the other forms.
  * Host-side query, no CUDA call. */
 int elbm_kernel_form(const elbm_solver* s, int* variant);
 

@@ -126,12 +126,14 @@ inline size_t cluster_smem(const Solver& s)
     return ((2 * band + 2) * 4 + 18 * band * storage_bytes(s.storage)) * s.nx;
 }
 
-// Grids the cluster takes: the band in shared memory, and at most kClMaxNodes nodes a
-// block.  us per step, cluster against march: 64 x 64 1.6 / 4.1,
-// 96 x 96 (1152 nodes a block) 3.1 / 4.15 FP32 and 2.8 / 4.2 FP16, 128 x 128 (2048)
-// 4.4 / 4.2 and 3.9 / 4.4, 160 x 100 4.3 / 4.2.
+// Grids the cluster takes: at most kClMaxNodes nodes a block.  us per step, cluster against
+// march: 64 x 64 1.6 / 4.1, 96 x 96 (1152 nodes a block) 2.95 / 4.1 FP32 and 2.75 / 4.3
+// FP16, 192 x 64 (1536) 3.35 / 4.1 and 3.15 / 4.35, 128 x 128 (2048) 4.4 / 4.2 and 3.9 / 4.4,
+// 160 x 100 (2080) 4.3 / 4.2.
 constexpr int kClMaxNodes = 3 * kClThreads;
-constexpr size_t kClMaxSmem = 220 * 1024;
+// ... whose shared memory is largest in FP32 with one row of them a block (cluster_smem()).
+constexpr size_t kClMaxSmem = (size_t)kClMaxNodes * (4 * 4 + 18 * 4);
+static_assert(kClMaxSmem <= 227 * 1024, "a band must fit the shared memory of a block");
 
 // Launch configuration of the cluster of s.
 struct ClusterLaunch {
@@ -187,7 +189,7 @@ inline int cluster_min_steps(const Solver& s)
 // Whether a call of nsteps steps of s takes the cluster.
 inline bool cluster_d2q9_applies(const Solver& s, int nsteps)
 {
-    if (s.D != 2 || (long long)cluster_band(s) * s.nx > kClMaxNodes || cluster_smem(s) > kClMaxSmem) return false;
+    if (s.D != 2 || (long long)cluster_band(s) * s.nx > kClMaxNodes) return false;
     if (nsteps < cluster_min_steps(s)) return false;
     switch (s.storage) {
         case ELBM_F32: return cluster_fits<ELBM_F32>(s);

@@ -35,20 +35,17 @@ __device__ __forceinline__ double red_warp(int k, double v)
     return k == 9 ? warp_min(v) : k == 11 ? warp_max(v) : warp_sum(v);
 }
 
-// Reduce the first NQ of ELBM_NRED FP64 accumulators over the block's first 8
-// warps (every thread of the block takes part in the barrier): warp shuffles,
-// then one shared-memory stage.
+// Reduce the first NQ of ELBM_NRED FP64 accumulators over the block (kBlock threads):
+// warp shuffles, then one shared-memory stage.
 template <int NQ>
 __device__ __forceinline__ void block_reduce(const double* acc, double* out)
 {
     __shared__ double sh[kBlock / 32][NQ];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp < kBlock / 32) {
 #pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-            const double v = red_warp(k, acc[k]);
-            if (lane == 0) sh[warp][k] = v;
-        }
+    for (int k = 0; k < NQ; ++k) {
+        const double v = red_warp(k, acc[k]);
+        if (lane == 0) sh[warp][k] = v;
     }
     __syncthreads();
     if (threadIdx.x < NQ) {

@@ -55,8 +55,8 @@ cudaError_t step_fused_impl(const Solver& s, int parity, unsigned long long* pro
 }
 
 // Single-pass kernel a step of s launches (the arrays are 16-byte aligned, as
-// the stream-ordered allocator returns them): 1 TMEM (32 x 16 tiles), 2 TMA
-// (32 x 8 tiles), 3 cp.async-fed; 4 the D2Q9 row march.  Walls and the
+// the stream-ordered allocator returns them): 1 TMEM (64 x 8 or 32 x 16
+// tiles), 2 TMA (32 x 8 tiles), 3 cp.async-fed; 4 D2Q9 (row march, cluster).  Walls and the
 // body force run in the TMEM kernel only.
 int single_pass_variant(const Solver& s)
 {

@@ -19,7 +19,6 @@
 namespace elbm {
 
 constexpr int kTileX = 32, kTileY = 8;   // kTileX * kTileY == kBlock
-constexpr int kHalo = 2 * kTileX + 2 * kTileY;
 
 // Planes per segment of a D3Q27 single-pass launch.  A block marches through
 // one tile column's segment of z planes and reads two planes more than it

@@ -271,17 +271,16 @@ cudaError_t step_two_pass_impl(const Solver& s, int parity, long long* launches)
     // walls and body force: the kernels of bounded_step.cuh (own translation units)
     if (p.walls_y || p.forced) return step_bounded_impl<D>(s, parity, launches);
     const dim3 grid((unsigned)((s.N + kBlock - 1) / kBlock));
-    const dim3 cgrid = grid;
     ELBM_DISPATCH_STORAGE(s.storage, {
         if (p.eq_mode == 2) {
-            if (parity == 0) k_collide<D, ST, 0, true><<<cgrid, kBlock, 0, s.stream>>>(p);
-            else k_collide<D, ST, 1, true><<<cgrid, kBlock, 0, s.stream>>>(p);
+            if (parity == 0) k_collide<D, ST, 0, true><<<grid, kBlock, 0, s.stream>>>(p);
+            else k_collide<D, ST, 1, true><<<grid, kBlock, 0, s.stream>>>(p);
         } else if (parity == 0) {
             if (p.eq_mode == 0) { k_anomaly<D, ST, 0><<<grid, kBlock, 0, s.stream>>>(p); ++*launches; }
-            k_collide<D, ST, 0><<<cgrid, kBlock, 0, s.stream>>>(p);
+            k_collide<D, ST, 0><<<grid, kBlock, 0, s.stream>>>(p);
         } else {
             if (p.eq_mode == 0) { k_anomaly<D, ST, 1><<<grid, kBlock, 0, s.stream>>>(p); ++*launches; }
-            k_collide<D, ST, 1><<<cgrid, kBlock, 0, s.stream>>>(p);
+            k_collide<D, ST, 1><<<grid, kBlock, 0, s.stream>>>(p);
         }
         ++*launches;
     });

@@ -262,8 +262,8 @@ class Solver:
     @property
     def kernel_form(self):
         """(form, variant) of the next step: form 1 two-pass, 2 graph-pipelined,
-        3 single pass; variant (form 3) 1 TMEM, 2 TMA, 3 cp.async-fed, 4 the
-        D2Q9 row march."""
+        3 single pass; variant (form 3) 1 TMEM, 2 TMA, 3 cp.async-fed, 4 D2Q9
+        (row march, and the cluster for several steps of a small grid)."""
         v = ctypes.c_int()
         form = load().elbm_kernel_form(self._h, ctypes.byref(v))
         if form < 0:

@@ -50,9 +50,9 @@ def test_segment_depths_of_eight_row_tiles_bitwise(n):
     assert np.array_equal(populations(elbm.D3Q27, n, elbm.F32, 3, (3,)), want)
 
 
-# tiles of the reduction are 32 x 8 nodes, the mode sums take 32 x 64: grids
-# inside one tile, one node past it, and ragged along every axis; one array at
-# both streaming parities
+# the gradient pass takes four nodes at once where rows allow it, the mode sums 32 x 64
+# nodes of a plane: grids inside that, one node past it, and ragged along every axis;
+# one array at both streaming parities
 @pytest.mark.parametrize("lattice,n", [(elbm.D3Q27, (5, 3, 70)), (elbm.D3Q27, (33, 9, 3)), (elbm.D3Q27, (97, 65, 4)),
                                        (elbm.D2Q9, (33, 5)), (elbm.D2Q9, (300, 130))])
 @pytest.mark.parametrize("steps,walls", [(0, False), (1, False), (1, True), (2, True)])
