@@ -231,14 +231,18 @@ __device__ __forceinline__ void collide_node(const StepParams& p, int cell)
 
 // Where the register form is the faster one: 16-bit storage, D2Q9, unshifted FP32 and
 // the periodic second-order equilibrium; not with the general body force, whose
-// increment leaves no registers.  us per two-pass step, registers against stage,
-// 135 x 121 x 150: FP16 125 / 136, FP32 161 / 161, FP32-shift 167 / 158; walls and x
-// force FP16 209 / 217, FP32 165 / 178, FP32-shift 200 / 190; second order FP16 76 / 93,
-// FP32-shift 93 / 102 (with walls 136 / 125); D2Q9 2048^2 FP32 95 / 102.
+// increment leaves no registers, nor for D3Q27 in 16 bits with the second-order
+// equilibrium between walls, which spills.  us per two-pass step, registers against stage,
+// 135 x 121 x 150: FP16 125 / 136, FP32 161 / 161, FP32-shift 167 / 158; walls and x force
+// FP16 209 / 217, FP32 165 / 178, FP32-shift 200 / 190; second order FP16 76 / 93, FP32-shift
+// 93 / 102; second order, walls and x force FP32 99 / 110, FP16 126 / 118, BF16 126 / 121,
+// FP32-shift 136 / 125; D2Q9 2048^2 FP32 95 / 102, with those options FP32 61 / 65, FP16
+// 50 / 62.
 template <int D, int ST, bool POLY, bool BC, bool FX>
 __host__ __device__ constexpr bool collide_in_registers()
 {
     if (BC && !FX) return false;
+    if (D == 3 && POLY && BC && sizeof(typename Storage<ST>::T) == 2) return false;
     return D == 2 || sizeof(typename Storage<ST>::T) == 2 || ST == ELBM_F32 || (POLY && !BC);
 }
 template <int D, int ST, bool POLY = false, bool BC = false, bool FX = false>

@@ -207,3 +207,17 @@ def test_single_pass_channel_against_oracle(storage, u_ref):
     (_, ug), (_, uo) = run_pair(elbm.D3Q27, TMEM_N, CHANNEL_LAM, CHANNEL_T, 0.02, rho, u, 201, storage,
                                 force=(2e-5, 0.0, 0.0), kernel=3, u_ref=u_ref)
     assert rel_linf(ug, uo) <= TOL[storage]
+
+
+@pytest.mark.parametrize("storage", [elbm.F32, elbm.F32_SHIFT, elbm.F16_SHIFT, elbm.BF16_SHIFT])
+@pytest.mark.parametrize("equilibrium", [0, 1, 2])
+@pytest.mark.parametrize("steps", [4, 5])
+def test_d3q27_channel_with_each_equilibrium(storage, equilibrium, steps):
+    """Walls and the x force in two passes, every storage and equilibrium (each
+    its own collision kernel), after an even and an odd step."""
+    rho, u = inputs.channel(CHANNEL_N, (1.0, 1.0, 1.0), u_center=0.05, perturbation=0.05, seed=1)
+    (rg, ug), (ro, uo) = run_pair(elbm.D3Q27, CHANNEL_N, (1.0, 1.0, 1.0), 1 / 3, 0.02, rho, u, steps, storage,
+                                  force=(2e-5, 0.0, 0.0), equilibrium=equilibrium)
+    tol = TOL.get(storage, 2e-2)
+    assert rel_linf(ug, uo) <= tol
+    assert np.abs(rg - ro).max() <= tol
