@@ -82,7 +82,9 @@ MEASURED_TRAFFIC = {("36d3ed5701ac3c47", "f32s", 0): 5.689e9, ("36d3ed5701ac3c47
                     # 217.07 B/node at 192^3, the same kernel (the header's documentation changed), x 256^3
                     ("fd488168e5bc7bf9", "f32s", 3): 3.642e9,
                     # 215.4 B/node at 192^3 with 64-wide tiles and the paired relaxation, x 256^3
-                    ("b45dddd09c6541c1", "f32s", 3): 3.614e9}
+                    ("b45dddd09c6541c1", "f32s", 3): 3.614e9,
+                    # 215.65 B/node at 192^3, the same kernel (two-pass 338.5)
+                    ("6c03ec4c13b5ac5c", "f32s", 3): 3.618e9, ("6c03ec4c13b5ac5c", "f32s", 1): 5.679e9}
 
 
 # The sources the step kernels' device code and launch shapes come from (the

@@ -112,8 +112,8 @@ struct TmemLayout {
 // in p it computes the same bits as BC = false.
 // PB != 0: the grid may be any; the tile's last columns and rows beyond it are
 // idle, the ring closes around the ones it has, and the four warps of the loading
-// warpgroup copy the tile with cp.async, a quarter of the populations each (no
-// tensor maps: rows need not start on 16 bytes).
+// warpgroup copy the tile and its ring with cp.async, a quarter of the populations
+// each (no tensor maps: rows need not start on 16 bytes).
 template <int ST, int TX, int NT, bool BC, bool FX = false, int PB = 0>
 __device__ __forceinline__ void tmem_tile_step(const CUtensorMap* tm_tile, const CUtensorMap* tm_row,
                                                const StepParams& p, void* dst, int x0, int y0, int z0, int z1,
